@@ -1057,9 +1057,11 @@ int hs_measure(hs_lattice *h, hs_measurement *out) {
     PassArgs a = base_args(h);
     a.n_colours = 1;
     a.pass = 0;
+    a.colour = 1;  // the sc kernel's work items: bonds are counted at colour 1
     a.finish = 1;
     a.accumulate = 0;
-    HS_CUDA(hs::launch_measure(h->precision, h->L, a, h->n_blocks, h->stream));
+    a.n_blocks = hs::measure_blocks(h->L, h->n_sm, h->max_blocks);
+    HS_CUDA(hs::launch_measure(h->precision, h->L, a, a.n_blocks, h->stream));
     double last[8], accepted = 0.0;
     HS_CUDA(cudaMemcpyAsync(last, h->acc->last, sizeof(last), cudaMemcpyDeviceToHost, h->stream));
     HS_CUDA(cudaMemcpyAsync(&accepted, &h->acc->accepted, sizeof(double), cudaMemcpyDeviceToHost, h->stream));

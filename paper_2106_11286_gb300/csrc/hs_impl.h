@@ -154,7 +154,9 @@ cudaError_t launch_gather_sites(int precision, const Layout &L, int64_t n, const
                                 cudaStream_t s);
 cudaError_t launch_scatter(int precision, const Layout &L, const double *d_xyz, cudaStream_t s);
 cudaError_t launch_gather(int precision, const Layout &L, double *d_xyz, cudaStream_t s);
+// Standalone measurement: a.colour = 1, a.n_blocks = n_blocks = measure_blocks(...).
 cudaError_t launch_measure(int precision, const Layout &L, const PassArgs &a, int n_blocks, cudaStream_t s);
+int measure_blocks(const Layout &L, int n_sm, int max_blocks);
 // Fold ring slots 0 .. n_slots-1 (sweeps of a.n_colours passes each, in sweep
 // order) into the accumulator: one CTA per slot sums it, then one thread
 // applies the totals in order.  1 <= n_slots <= kRingMax.

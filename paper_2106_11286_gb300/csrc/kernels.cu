@@ -454,75 +454,268 @@ __global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (W > 0 ? 4 : 5)) ta
 }
 
 // ----------------------------------------------------------------- measure
-// Standalone Eq. 1 / Eq. 2 of the current state in FP64: every site adds
-// -J/2 S_i.h_i - K (S_i.e)^2, so each bond is counted once overall.
-template <int P>
-__global__ void __launch_bounds__(kBlock) sc_measure_kernel(const PassArgs a, const void *planes) {
-    pdl_enter();
-    using S = typename Tr<P>::S;
-    const S *pl = (const S *)planes;
-    const int Lh = a.Lh, Ly = a.Ly, Lz = a.Lz;
-    const int64_t plane = (int64_t)Lz * Ly * Lh;
-    double accE = 0, accX = 0, accY = 0, accZ = 0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < 2 * plane; t += stride) {
-        const int c = (int)(t / plane);
-        const int64_t idx = t - c * plane;
-        const int xh = (int)(idx % Lh);
-        const int64_t row = idx / Lh;
-        const int y = (int)(row % Ly), z = (int)(row / Ly);
-        const int p = (y + z + c) & 1;
-        const S *me = pl + (int64_t)(3 * c) * plane;
-        const S *ot = pl + (int64_t)(3 * (1 - c)) * plane;
-        const int xm = p ? xh : (xh == 0 ? Lh - 1 : xh - 1);
-        const int xp = p ? (xh == Lh - 1 ? 0 : xh + 1) : xh;
-        const int ym = (y == 0) ? Ly - 1 : y - 1, yp = (y == Ly - 1) ? 0 : y + 1;
-        const int zm = (z == 0) ? Lz - 1 : z - 1, zp = (z == Lz - 1) ? 0 : z + 1;
-        const int64_t nb[6] = {row * Lh + xm,
-                               row * Lh + xp,
-                               ((int64_t)z * Ly + ym) * Lh + xh,
-                               ((int64_t)z * Ly + yp) * Lh + xh,
-                               ((int64_t)zm * Ly + y) * Lh + xh,
-                               ((int64_t)zp * Ly + y) * Lh + xh};
-        double s[3], h[3] = {0.0, 0.0, 0.0};
-        for (int q = 0; q < 3; ++q) {
-            s[q] = (double)to_c(me[q * plane + idx]);
-            for (int k = 0; k < 6; ++k) h[q] += (double)to_c(ot[q * plane + nb[k]]);
-        }
-        const double se = s[0] * a.e[0] + s[1] * a.e[1] + s[2] * a.e[2];
-        accE += -0.5 * a.J * (s[0] * h[0] + s[1] * h[1] + s[2] * h[2]) - a.K * se * se;
-        if (a.tensor) accE -= quad64(s[0], s[1], s[2], a.A);
-        accX += s[0];
-        accY += s[1];
-        accZ += s[2];
-    }
-    write_partials<double, true>(a, accE, accX, accY, accZ, 0u);
+// Standalone Eq. 1 / Eq. 2 of the current state to FP64 accuracy.
+//
+// FP32 / FP16 storage works in unevaluated pairs of floats: every addition
+// keeps its rounding error (TwoSum, Knuth, The Art of Computer Programming
+// vol. 2, 4.2.2) and every product its remainder (one fma), so a site's share
+// carries 48 bits and a thread's sums lose nothing that FP64 sums of the same
+// numbers would keep; the FP64 pipe, which issues 2 instructions per cycle
+// per SM against 128 for FP32, is left with one conversion per thread.  The
+// plain FP64 form, 45 FP64 instructions and 21 conversions a site, took
+// 2059 us at 256^3 and 12177 us at 464^3 FP32; a whole case of ten 464^3
+// sweeps, a measurement and the spins' read-back went from 19.08 to 7.35 ms
+// with this one (FP16 19.30 to 7.80, the 3.1 M-site nanoparticle 1.50 to 1.17).
+// On the sc stencil every bond is counted once, at its colour-1 site, from the
+// vector loads of the sweep's work items; colour 0 adds its own spins only.
+template <typename T>
+__device__ __forceinline__ T sub_exact(T a, T b) { return f_fma(splat<T>(-1.0f), b, a); }  // a - b, one rounding
+
+// a + v with the rounding error added to lo
+template <typename T>
+__device__ __forceinline__ void two_sum(T &a, T &lo, T v) {
+    const T s = f_add(a, v);
+    const T bb = sub_exact(s, a);
+    const T e = f_add(sub_exact(a, sub_exact(s, bb)), sub_exact(v, bb));
+    a = s;
+    lo = f_add(lo, e);
 }
 
+// sum += s (hh + hl), the product's remainder kept in lo
+template <typename T>
+__device__ __forceinline__ void two_prod_add(T &sum, T &lo, T s, T hh, T hl) {
+    const T p = f_mul(s, hh);
+    const T r = f_fma(s, hh, f_mul(splat<T>(-1.0f), p));
+    lo = f_add(lo, f_fma(s, hl, r));
+    two_sum(sum, lo, p);
+}
+
+// Sums of one thread: bonds, (S.e)^2 and the spin components, as pairs.
+template <typename T>
+struct PairSums {
+    T b, bl, k, kl, m[3], ml[3];
+    __device__ __forceinline__ PairSums() {
+        b = bl = k = kl = splat<T>(0.0f);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) m[q] = ml[q] = splat<T>(0.0f);
+    }
+};
+__device__ __forceinline__ double wide_sum(float h, float l) { return (double)h + (double)l; }
+__device__ __forceinline__ double wide_sum(float2 h, float2 l) {
+    return wide_sum(h.x, l.x) + wide_sum(h.y, l.y);
+}
+
+template <typename T, typename S, int V>
+__device__ __forceinline__ T lanes(const Vec<S, V> &v, int j) {
+    if constexpr (std::is_same<T, float2>::value)
+        return make_float2(to_c(v.v[2 * j]), to_c(v.v[2 * j + 1]));
+    else
+        return to_c(v.v[j]);
+}
+
+// quotient of a work-item or row index, beyond FastDiv's range by division
+__device__ __forceinline__ uint32_t div_any(const FastDiv &d, uint32_t n) {
+    return n < 0x80000000u ? d.div(n) : n / d.d;
+}
+
+// The on-site terms of one site in FP64 (an easy axis other than z, or the tensor): K (S.e)^2 + S^T A S.
+__device__ __forceinline__ double onsite64(const PassArgs &a, double x, double y, double z) {
+    const double se = x * a.e[0] + y * a.e[1] + z * a.e[2];
+    const double k = a.K * se * se;
+    return a.tensor ? k + quad64(x, y, z, a.A) : k;
+}
+
+// GEN: the on-site terms need FP64 (onsite64); else S.e = S_z or K = 0.
+template <int P, int V, bool GEN>
+__global__ void __launch_bounds__(kBlock) sc_measure_kernel(const PassArgs a, const void *planes, uint32_t n_items) {
+    using S = typename Tr<P>::S;
+    using VT = Vec<S, V>;
+    const S *pl = (const S *)planes;
+    const int64_t plane = (int64_t)a.Lz * a.Ly * a.Lh;
+    const S *const c0[3] = {pl, pl + plane, pl + 2 * plane};
+    const S *const c1[3] = {pl + 3 * plane, pl + 4 * plane, pl + 5 * plane};
+    const uint32_t stride = gridDim.x * blockDim.x;
+    const uint32_t t0 = blockIdx.x * blockDim.x + threadIdx.x;
+    double accG = 0.0;
+    // colour-1 work item t (a.colour = 1): its own spins and their neighbours'
+    auto load = [&](uint32_t t, StencilItem<P, V> &it) {
+        const uint32_t nxv = a.Lh / V;
+        const uint32_t row = div_any(a.div_nxv, t);
+        const uint32_t z = div_any(a.div_ly, row);
+        load_item_at<P, V>(a, row - z * a.Ly, z, t - row * nxv, c1, c0, it);
+    };
+    if constexpr (P == HS_FP64) {
+        double b = 0, k = 0, m[3] = {0, 0, 0};
+        auto own = [&](const VT (&s)[3]) {
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) m[q] += s[q].v[j];
+                if (GEN)
+                    accG += onsite64(a, s[0].v[j], s[1].v[j], s[2].v[j]);
+                else
+                    k = fma(s[2].v[j], s[2].v[j], k);
+            }
+        };
+        for (uint64_t t = t0; t < n_items; t += stride) {
+            VT s[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) s[q] = *reinterpret_cast<const VT *>(c0[q] + t * V);
+            own(s);
+        }
+        for (uint64_t t = t0; t < n_items; t += stride) {
+            StencilItem<P, V> it;
+            load((uint32_t)t, it);
+            double h[3][V];
+            item_fields<P, V>(it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, h);
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) b = fma(it.s[q].v[j], h[q][j], b);
+            own(it.s);
+        }
+        write_partials<double, true>(a, -a.J * b - (GEN ? accG : (a.K == 0.0 ? 0.0 : a.K * k)), m[0], m[1], m[2], 0u);
+    } else {
+        using T = typename std::conditional<(V >= 2), float2, float>::type;
+        constexpr int W = V >= 2 ? V / 2 : 1;  // lane groups of an item
+        PairSums<T> A;
+        auto own = [&](const VT (&s)[3]) {
+#pragma unroll
+            for (int j = 0; j < W; ++j) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) two_sum(A.m[q], A.ml[q], lanes<T>(s[q], j));
+                if (!GEN) {
+                    const T z = lanes<T>(s[2], j);
+                    two_prod_add(A.k, A.kl, z, z, splat<T>(0.0f));
+                }
+            }
+            if (GEN)
+#pragma unroll
+                for (int j = 0; j < V; ++j) accG += onsite64(a, to_c(s[0].v[j]), to_c(s[1].v[j]), to_c(s[2].v[j]));
+        };
+        for (uint64_t t = t0; t < n_items; t += stride) {
+            VT s[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) s[q] = *reinterpret_cast<const VT *>(c0[q] + t * V);
+            own(s);
+        }
+        for (uint64_t t = t0; t < n_items; t += stride) {
+            StencilItem<P, V> it;
+            load((uint32_t)t, it);
+#pragma unroll
+            for (int j = 0; j < W; ++j)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    // the x neighbours: the same row's vector and its edge element on the side that p picks
+                    T x;
+                    if constexpr (V >= 2) {
+                        const float prev = j == 0 ? it.ed[q] : to_c(it.o[q].v[j == 0 ? 0 : 2 * j - 1]);
+                        const float next = j == W - 1 ? it.ed[q] : to_c(it.o[q].v[j == W - 1 ? 0 : 2 * j + 2]);
+                        x = it.p ? make_float2(to_c(it.o[q].v[2 * j + 1]), next)
+                                 : make_float2(prev, to_c(it.o[q].v[2 * j]));
+                    } else {
+                        x = it.ed[q];
+                    }
+                    T h = lanes<T>(it.o[q], j), hl = splat<T>(0.0f);
+                    two_sum(h, hl, x);
+                    two_sum(h, hl, lanes<T>(it.nym[q], j));
+                    two_sum(h, hl, lanes<T>(it.nyp[q], j));
+                    two_sum(h, hl, lanes<T>(it.nzm[q], j));
+                    two_sum(h, hl, lanes<T>(it.nzp[q], j));
+                    two_prod_add(A.b, A.bl, lanes<T>(it.s[q], j), h, hl);
+                }
+            own(it.s);
+        }
+        double b = wide_sum(A.b, A.bl), k = wide_sum(A.k, A.kl);
+        double m[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) m[q] = wide_sum(A.m[q], A.ml[q]);
+        // beyond FP32's range (no unit vectors): the same sums in FP64
+        if (!(isfinite(b) && isfinite(k) && isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]))) {
+            b = k = m[0] = m[1] = m[2] = accG = 0.0;
+            for (uint64_t t = t0; t < n_items; t += stride) {
+                StencilItem<P, V> it;
+                load((uint32_t)t, it);
+                for (int j = 0; j < V; ++j)
+                    for (int c = 0; c < 2; ++c) {
+                        double s[3];
+                        for (int q = 0; q < 3; ++q) {
+                            s[q] = (double)to_c(c == 0 ? c0[q][t * V + j] : it.s[q].v[j]);
+                            m[q] += s[q];
+                            if (c == 0) continue;
+                            const double x = it.p ? (double)(j == V - 1 ? it.ed[q] : to_c(it.o[q].v[j + 1]))
+                                                  : (double)(j == 0 ? it.ed[q] : to_c(it.o[q].v[j - 1]));
+                            b += s[q] * ((double)to_c(it.o[q].v[j]) + x + (double)to_c(it.nym[q].v[j]) +
+                                         (double)to_c(it.nyp[q].v[j]) + (double)to_c(it.nzm[q].v[j]) +
+                                         (double)to_c(it.nzp[q].v[j]));
+                        }
+                        if (GEN)
+                            accG += onsite64(a, s[0], s[1], s[2]);
+                        else
+                            k += s[2] * s[2];
+                    }
+            }
+        }
+        write_partials<double, true>(a, -a.J * b - (GEN ? accG : (a.K == 0.0 ? 0.0 : a.K * k)), m[0], m[1], m[2], 0u);
+    }
+}
+
+// Neighbour table: every site adds -J/2 S_i.h_i and its on-site terms, so each bond is counted once overall.
 template <int P>
 __global__ void __launch_bounds__(kBlock) table_measure_kernel(const PassArgs a, int64_t n_present) {
-    pdl_enter();
     using S = typename Tr<P>::S;
+    using C = typename Tr<P>::C;
     using S4 = Vec<S, 4>;
     const S4 *spins = reinterpret_cast<const S4 *>(a.spins4);
-    double accE = 0, accX = 0, accY = 0, accZ = 0;
+    const bool onsite = a.K != 0.0 || a.tensor;
+    double b = 0, g = 0, m[3] = {0, 0, 0};
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_present; i += stride) {
-        double h[3] = {0.0, 0.0, 0.0};
-        for (int k = 0; k < a.width; ++k) {
-            const S4 n = spins[a.nbr[(int64_t)k * a.n_pad + i]];
-            for (int q = 0; q < 3; ++q) h[q] += (double)to_c(n.v[q]);
-        }
+    PairSums<float> A;
+    for (int64_t i = t0; i < n_present; i += stride) {
+        C h[3] = {C(0), C(0), C(0)}, hl[3] = {C(0), C(0), C(0)};
         const S4 sv = spins[i];
-        const double s0 = to_c(sv.v[0]), s1 = to_c(sv.v[1]), s2 = to_c(sv.v[2]);
-        const double se = s0 * a.e[0] + s1 * a.e[1] + s2 * a.e[2];
-        accE += -0.5 * a.J * (s0 * h[0] + s1 * h[1] + s2 * h[2]) - a.K * se * se;
-        if (a.tensor) accE -= quad64(s0, s1, s2, a.A);
-        accX += s0;
-        accY += s1;
-        accZ += s2;
+#pragma unroll 4
+        for (int k = 0; k < a.width; ++k) {
+            const S4 n = spins[__ldg(a.nbr + (int64_t)k * a.n_pad + i)];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                if constexpr (P == HS_FP64)
+                    h[q] += n.v[q];
+                else
+                    two_sum(h[q], hl[q], to_c(n.v[q]));
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const C s = to_c(sv.v[q]);
+            if constexpr (P == HS_FP64) {
+                b = fma(s, h[q], b);
+                m[q] += s;
+            } else {
+                two_prod_add(A.b, A.bl, s, h[q], hl[q]);
+                two_sum(A.m[q], A.ml[q], s);
+            }
+        }
+        if (onsite) g += onsite64(a, to_c(sv.v[0]), to_c(sv.v[1]), to_c(sv.v[2]));
     }
-    write_partials<double, true>(a, accE, accX, accY, accZ, 0u);
+    if constexpr (P != HS_FP64) {
+        b = wide_sum(A.b, A.bl);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) m[q] = wide_sum(A.m[q], A.ml[q]);
+        if (!(isfinite(b) && isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]))) {  // beyond FP32's range
+            b = m[0] = m[1] = m[2] = 0.0;
+            for (int64_t i = t0; i < n_present; i += stride)
+                for (int q = 0; q < 3; ++q) {
+                    double h = 0.0;
+                    for (int k = 0; k < a.width; ++k)
+                        h += (double)to_c(spins[a.nbr[(int64_t)k * a.n_pad + i]].v[q]);
+                    b += (double)to_c(spins[i].v[q]) * h;
+                    m[q] += (double)to_c(spins[i].v[q]);
+                }
+        }
+    }
+    write_partials<double, true>(a, -0.5 * a.J * b - g, m[0], m[1], m[2], 0u);
 }
 
 // ----------------------------------------------------------------- fold
@@ -1007,23 +1200,47 @@ cudaError_t launch_pass(int precision, const Layout &L, const PassArgs &a, int n
     }
 }
 
-cudaError_t launch_measure(int precision, const Layout &L, const PassArgs &a, int n_blocks, cudaStream_t s) {
-    if (L.structured) {
-        switch (precision) {
-        case HS_FP64: sc_measure_kernel<HS_FP64><<<n_blocks, kBlock, 0, s>>>(a, L.planes); break;
-        case HS_FP32: sc_measure_kernel<HS_FP32><<<n_blocks, kBlock, 0, s>>>(a, L.planes); break;
-        case HS_FP16: sc_measure_kernel<HS_FP16><<<n_blocks, kBlock, 0, s>>>(a, L.planes); break;
-        default: return cudaErrorInvalidValue;
-        }
-    } else {
-        switch (precision) {
-        case HS_FP64: table_measure_kernel<HS_FP64><<<n_blocks, kBlock, 0, s>>>(a, L.n_present); break;
-        case HS_FP32: table_measure_kernel<HS_FP32><<<n_blocks, kBlock, 0, s>>>(a, L.n_present); break;
-        case HS_FP16: table_measure_kernel<HS_FP16><<<n_blocks, kBlock, 0, s>>>(a, L.n_present); break;
-        default: return cudaErrorInvalidValue;
-        }
+template <int P, int V>
+static void measure_sc(const PassArgs &a, const Layout &L, int n_blocks, cudaStream_t s) {
+    const uint32_t n_items = (uint32_t)((int64_t)L.nz * L.Ly * (L.Lh / V));
+    if (a.tensor || (a.K != 0.0 && !a.zaxis))
+        sc_measure_kernel<P, V, true><<<n_blocks, kBlock, 0, s>>>(a, L.planes, n_items);
+    else
+        sc_measure_kernel<P, V, false><<<n_blocks, kBlock, 0, s>>>(a, L.planes, n_items);
+}
+
+template <int P>
+static bool measure_p(const Layout &L, const PassArgs &a, int n_blocks, cudaStream_t s) {
+    if (!L.structured) {
+        table_measure_kernel<P><<<n_blocks, kBlock, 0, s>>>(a, L.n_present);
+        return true;
     }
-    return cudaGetLastError();
+    switch (L.vec) {
+    case 1: measure_sc<P, 1>(a, L, n_blocks, s); return true;
+    case 2: measure_sc<P, 2>(a, L, n_blocks, s); return true;
+    case 4: if constexpr (P != HS_FP64) { measure_sc<P, 4>(a, L, n_blocks, s); return true; } break;
+    case 8: if constexpr (P == HS_FP16) { measure_sc<P, 8>(a, L, n_blocks, s); return true; } break;
+    default: break;
+    }
+    return false;
+}
+
+// CTAs of a measurement: enough threads to hide the loads of its short items (two sites of FP64 to eight of
+// FP16), as many as the partials buffer holds at most.
+int measure_blocks(const Layout &L, int n_sm, int max_blocks) {
+    const int64_t items = L.structured ? pass_items(L) : L.n_present;
+    return std::min(grid_for(items, n_sm * 6), max_blocks);
+}
+
+cudaError_t launch_measure(int precision, const Layout &L, const PassArgs &a, int n_blocks, cudaStream_t s) {
+    bool known = false;
+    switch (precision) {
+    case HS_FP64: known = measure_p<HS_FP64>(L, a, n_blocks, s); break;
+    case HS_FP32: known = measure_p<HS_FP32>(L, a, n_blocks, s); break;
+    case HS_FP16: known = measure_p<HS_FP16>(L, a, n_blocks, s); break;
+    default: break;
+    }
+    return known ? cudaGetLastError() : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_init(int precision, const Layout &L, int mode, const double e[3], uint32_t key0, uint32_t key1,
