@@ -807,8 +807,8 @@ __global__ void table_init_kernel(void *spins4, const uint32_t *nat, int64_t n_p
 }
 
 template <int P>
-__global__ void sc_convert_kernel(void *planes, double *xyz, int Lx, int Ly, int nz, int Lz_arr, int z_off, int z0,
-                                  int Lh, int to_layout) {
+__global__ void sc_scatter_kernel(void *planes, const double *xyz, int Lx, int Ly, int nz, int Lz_arr, int z_off,
+                                  int z0, int Lh) {
     using S = typename Tr<P>::S;
     S *pl = (S *)planes;
     const int64_t plane = (int64_t)Lz_arr * Ly * Lh;
@@ -819,13 +819,76 @@ __global__ void sc_convert_kernel(void *planes, double *xyz, int Lx, int Ly, int
         const int y = (int)(r % Ly), z = (int)(r / Ly);
         const int c = (x + y + z + z0) & 1;
         const int64_t idx = (r + (int64_t)z_off * Ly) * Lh + (x >> 1);
-        for (int q = 0; q < 3; ++q) {
-            S *d = pl + (int64_t)(3 * c + q) * plane + idx;
-            if (to_layout)
-                *d = store_from_double<S>(xyz[3 * i + q]);
-            else
-                xyz[3 * i + q] = (double)to_c(*d);
+        for (int q = 0; q < 3; ++q) pl[(int64_t)(3 * c + q) * plane + idx] = store_from_double<S>(xyz[3 * i + q]);
+    }
+}
+
+// A float's value as a double, from its bit fields in the integer pipe: the
+// conversion instruction runs at the FP64 pipe's rate, 2 a cycle per SM.
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t b = __float_as_uint(f), e = b & 0x7F800000u, m = b & 0x7FFFFFFFu;
+    if (m != 0u && (e == 0u || e == 0x7F800000u)) return (double)f;  // subnormal, infinity, NaN
+    const uint32_t hi = m == 0u ? b : ((b & 0x80000000u) | ((m >> 3) + (896u << 20)));
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
+// The whole state in natural order, FP64.  V sites of each colour at one row
+// offset are 2 V consecutive sites; a CTA stages its kBlock such runs in
+// shared memory and stores them as consecutive 16-byte pairs (8-byte ones
+// where the caller's buffer is not 16-byte aligned), evict-first: the lattice
+// stays in L2 for the next sweep.  Bound by HBM (read once, 24 bytes a site
+// written: 3.6 GB at 464^3 FP32 in about 650 us); one thread per site with
+// three strided stores and 64-bit divisions took 1102 us there.
+template <int P, int V>
+__global__ void __launch_bounds__(kBlock) sc_export_kernel(const void *planes, double *xyz, int Ly, int64_t plane,
+                                                           int Lh, int z_off, int z0, FastDiv div_nxv, FastDiv div_ly,
+                                                           uint32_t n_vec, int aligned) {
+    using S = typename Tr<P>::S;
+    using C = typename Tr<P>::C;
+    using VT = Vec<S, V>;
+    __shared__ __align__(16) C st[kBlock * 6 * V];
+    const S *pl = (const S *)planes;
+    for (uint64_t t0 = (uint64_t)blockIdx.x * kBlock; t0 < n_vec; t0 += (uint64_t)gridDim.x * kBlock) {
+        const uint32_t cnt = (uint32_t)(n_vec - t0 < kBlock ? n_vec - t0 : kBlock);
+        if (threadIdx.x < cnt) {
+            const uint32_t t = (uint32_t)t0 + threadIdx.x;
+            const uint32_t row = div_any(div_nxv, t);
+            const uint32_t z = div_any(div_ly, row);
+            const uint32_t y = row - z * (uint32_t)Ly;
+            const int first = (int)((y + z + (uint32_t)z0) & 1u);  // the colour of even x in this row
+            const int64_t idx = (int64_t)t * V + (int64_t)z_off * Ly * Lh;
+            VT v[2][3];
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    v[c][q] = *reinterpret_cast<const VT *>(pl + (3 * (c ^ first) + q) * plane + idx);
+            C *d = st + threadIdx.x * 6 * V;
+            C out[6 * V];
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) out[6 * j + 3 * c + q] = to_c(v[c][q].v[j]);
+#pragma unroll
+            for (int k = 0; k < 3 * V; ++k)
+                *reinterpret_cast<Vec<C, 2> *>(d + 2 * k) = Vec<C, 2>{{out[2 * k], out[2 * k + 1]}};
         }
+        __syncthreads();
+        double *o = xyz + t0 * 6 * V;
+        for (uint32_t k = threadIdx.x; k < cnt * 3 * V; k += kBlock) {
+            const Vec<C, 2> f = *reinterpret_cast<const Vec<C, 2> *>(st + 2 * k);
+            const double2 w = make_double2(widen(f.v[0]), widen(f.v[1]));
+            if (aligned) {
+                __stcs(reinterpret_cast<double2 *>(o) + k, w);
+            } else {
+                __stcs(o + 2 * k, w.x);
+                __stcs(o + 2 * k + 1, w.y);
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -1283,34 +1346,37 @@ cudaError_t launch_init(int precision, const Layout &L, int mode, const double e
     return cudaGetLastError();
 }
 
-static cudaError_t launch_convert(int precision, const Layout &L, double *xyz, int to_layout, cudaStream_t s) {
-    if (L.structured) {
-        const int g = grid_for(L.n_sites);
-        switch (precision) {
-        case HS_FP64:
-            sc_convert_kernel<HS_FP64><<<g, kBlock, 0, s>>>(L.planes, xyz, L.Lx, L.Ly, L.nz, L.Lz, L.slab ? 1 : 0, L.z0,
-                                                          L.Lh, to_layout);
-            break;
-        case HS_FP32:
-            sc_convert_kernel<HS_FP32><<<g, kBlock, 0, s>>>(L.planes, xyz, L.Lx, L.Ly, L.nz, L.Lz, L.slab ? 1 : 0, L.z0,
-                                                          L.Lh, to_layout);
-            break;
-        case HS_FP16:
-            sc_convert_kernel<HS_FP16><<<g, kBlock, 0, s>>>(L.planes, xyz, L.Lx, L.Ly, L.nz, L.Lz, L.slab ? 1 : 0, L.z0,
-                                                          L.Lh, to_layout);
-            break;
-        default: return cudaErrorInvalidValue;
-        }
-    } else {
-        const int g = grid_for(L.n_present);
-        switch (precision) {
-        case HS_FP64: table_convert_kernel<HS_FP64><<<g, kBlock, 0, s>>>(L.spins4, L.nat, L.n_present, xyz, to_layout); break;
-        case HS_FP32: table_convert_kernel<HS_FP32><<<g, kBlock, 0, s>>>(L.spins4, L.nat, L.n_present, xyz, to_layout); break;
-        case HS_FP16: table_convert_kernel<HS_FP16><<<g, kBlock, 0, s>>>(L.spins4, L.nat, L.n_present, xyz, to_layout); break;
-        default: return cudaErrorInvalidValue;
-        }
-    }
+template <int P>
+static cudaError_t table_convert(const Layout &L, double *xyz, int to_layout, cudaStream_t s) {
+    table_convert_kernel<P><<<grid_for(L.n_present), kBlock, 0, s>>>(L.spins4, L.nat, L.n_present, xyz, to_layout);
     return cudaGetLastError();
+}
+
+template <int P>
+static cudaError_t scatter_p(const Layout &L, double *xyz, cudaStream_t s) {
+    if (!L.structured) return table_convert<P>(L, xyz, 1, s);
+    sc_scatter_kernel<P><<<grid_for(L.n_sites), kBlock, 0, s>>>(L.planes, xyz, L.Lx, L.Ly, L.nz, L.Lz, L.slab ? 1 : 0,
+                                                                L.z0, L.Lh);
+    return cudaGetLastError();
+}
+
+template <int P, int V>
+static cudaError_t export_v(const Layout &L, double *xyz, cudaStream_t s) {
+    const int64_t n_vec = (int64_t)L.nz * L.Ly * (L.Lh / V);
+    sc_export_kernel<P, V><<<grid_for(n_vec, 152 * 8), kBlock, 0, s>>>(
+        L.planes, xyz, L.Ly, (int64_t)L.Lz * L.Ly * L.Lh, L.Lh, L.slab ? 1 : 0, L.z0, FastDiv((uint32_t)(L.Lh / V)),
+        FastDiv((uint32_t)L.Ly), (uint32_t)n_vec, (uintptr_t)xyz % 16 == 0 ? 1 : 0);
+    return cudaGetLastError();
+}
+
+// Vector width by what divides the row: four sites of FP32 / FP16, two of FP64 (16 bytes at most).
+template <int P>
+static cudaError_t gather_p(const Layout &L, double *xyz, cudaStream_t s) {
+    if (!L.structured) return table_convert<P>(L, xyz, 0, s);
+    if constexpr (P != HS_FP64)
+        if (L.Lh % 4 == 0) return export_v<P, 4>(L, xyz, s);
+    if (L.Lh % 2 == 0) return export_v<P, 2>(L, xyz, s);
+    return export_v<P, 1>(L, xyz, s);
 }
 
 cudaError_t launch_gather_sites(int precision, const Layout &L, int64_t n, const int64_t *d_sites, double *d_out,
@@ -1333,11 +1399,22 @@ cudaError_t launch_gather_sites(int precision, const Layout &L, int64_t n, const
 }
 
 cudaError_t launch_scatter(int precision, const Layout &L, const double *d_xyz, cudaStream_t s) {
-    return launch_convert(precision, L, const_cast<double *>(d_xyz), 1, s);
+    double *xyz = const_cast<double *>(d_xyz);
+    switch (precision) {
+    case HS_FP64: return scatter_p<HS_FP64>(L, xyz, s);
+    case HS_FP32: return scatter_p<HS_FP32>(L, xyz, s);
+    case HS_FP16: return scatter_p<HS_FP16>(L, xyz, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_gather(int precision, const Layout &L, double *d_xyz, cudaStream_t s) {
-    return launch_convert(precision, L, d_xyz, 0, s);
+    switch (precision) {
+    case HS_FP64: return gather_p<HS_FP64>(L, d_xyz, s);
+    case HS_FP32: return gather_p<HS_FP32>(L, d_xyz, s);
+    case HS_FP16: return gather_p<HS_FP16>(L, d_xyz, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace hs
