@@ -199,7 +199,7 @@ struct hs_lattice {
     uint64_t sweep = 0;
     int accumulate = 0;
     int64_t last_n_sweeps = 0;
-    double2 *sc_tab = nullptr;     // FP64: sin, cos(pi j / 1024) table of the trial orientation
+    ulonglong2 *sc_tab = nullptr;  // FP64: sine and cosine table of the trial orientation
     int tensor = 0;                // on-site anisotropy tensor term on
     double tA[6] = {0, 0, 0, 0, 0, 0};
     Layout L{};
@@ -685,16 +685,17 @@ int lattice_create(hs_lattice **out, int type, const int32_t dims[3], int period
     }
     if (st == HS_OK) st = h->alloc(&h->acc, sizeof(DevAccum));
     if (st == HS_OK && precision == HS_FP64) {
-        // sin, cos(pi j / 1024) for the FP64 trial's table lookup, from long double on the host
+        // sin, cos(pi j / 4096) in units of 2^-63 for the FP64 trial's table lookup, from long double on the host
         const long double pi = 3.141592653589793238462643383279502884L;
-        std::vector<double2> tab(2048);
+        std::vector<ulonglong2> tab(2048);
         for (int j = 0; j < 2048; ++j) {
-            const long double a = pi * (long double)j / 1024.0L;
-            tab[j] = make_double2((double)sinl(a), (double)cosl(a));
+            const long double a = pi * (long double)j / 4096.0L;
+            tab[j] = make_ulonglong2((unsigned long long)(sinl(a) * 0x1p63L + 0.5L),
+                                     (unsigned long long)(cosl(a) * 0x1p63L + 0.5L));
         }
-        st = h->alloc(&h->sc_tab, tab.size() * sizeof(double2));
+        st = h->alloc(&h->sc_tab, tab.size() * sizeof(ulonglong2));
         if (st == HS_OK) {
-            cudaError_t e = cudaMemcpy(h->sc_tab, tab.data(), tab.size() * sizeof(double2), cudaMemcpyHostToDevice);
+            cudaError_t e = cudaMemcpy(h->sc_tab, tab.data(), tab.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice);
             if (e != cudaSuccess) st = cuda_fail(e, "cudaMemcpy");
         }
     }
@@ -787,6 +788,12 @@ int run_pass(hs_lattice *h, PassArgs &a, uint32_t sweep, int c, bool deferred = 
     return HS_OK;
 }
 
+void set_beta(const hs_lattice *h, PassArgs &a, double beta) {
+    a.beta = beta;
+    a.fbeta = (float)beta;
+    a.fdelta = hs::decision_band(beta, h->p.J, h->p.K, h->L.structured ? 6 : h->L.width);
+}
+
 int check_beta(double beta) {
     if (!(beta >= 0.0) || !std::isfinite(beta)) return fail(HS_E_INVALID, "beta must be finite and >= 0");
     return HS_OK;
@@ -806,8 +813,7 @@ int hs_sweep(hs_lattice *h, double beta, int64_t n_sweeps) {
         return HS_OK;
     }
     PassArgs a = base_args(h);
-    a.beta = beta;
-    a.fbeta = (float)beta;
+    set_beta(h, a, beta);
     a.accumulate = h->accumulate;
     // sweep s writes ring slot s mod ring; each full ring, and the rest after
     // the loop, is folded into the accumulator in sweep order
@@ -889,8 +895,7 @@ int hs_sweep_pass_part(hs_lattice *h, double beta, int colour, int part) {
     }
     if (L.n_present > 0) {
         PassArgs a = base_args(h);
-        a.beta = beta;
-        a.fbeta = (float)beta;
+        set_beta(h, a, beta);
         // a slab always measures its fused sums (the observables of a lattice split into slabs come from
         // all slabs' sums); only accumulation adds its own moments
         a.accumulate = h->accumulate ? 1 : (L.slab ? 2 : 0);
@@ -1758,6 +1763,7 @@ int hs_batch_run(hs_batch *b, const double *betas, int64_t n_sweeps, int64_t n_e
         hs_lattice *h = b->members[r];
         b->host_members[r].fbeta = (float)betas[r];
         b->host_members[r].beta = betas[r];
+        b->host_members[r].fdelta = hs::decision_band(betas[r], h->p.J, h->p.K, 6);
         b->host_members[r].sweep0 = (uint32_t)h->sweep;
         h->last_n_sweeps = n_total;
     }

@@ -89,6 +89,7 @@ __device__ __forceinline__ PassArgs member_args(const BatchMember &m, int colour
     a.beta = m.beta;
     a.sc_tab = m.sc_tab;
     a.zaxis = m.zaxis;
+    a.fdelta = m.fdelta;
     a.key0 = m.key0;
     a.key1 = m.key1;
     a.replica = m.replica;
@@ -211,14 +212,15 @@ __device__ __forceinline__ void batch_pass(const BatchArgs &b, int s, int c) {
                 while (true) {
                     VT nym[3], nyp[3];
                     load_split_b<P, V, CG>(A, oth, nym, nyp);
-                    C h[3][V];
-                    item_fields<P, V>(A.o, nym, nyp, A.nzm, A.nzp, A.ed, A.f.p, h);
+                    typename ItemField<P, V>::T h;
+                    fields_of<P, V, true, false>(A.o, nym, nyp, A.nzm, A.nzp, A.ed, A.f.p, c, h);
                     VT sv[3] = {A.s[0], A.s[1], A.s[2]};
                     const uint32_t b0 = A.f.b0, site0 = A.f.site0, rank0 = A.f.rank0;
                     const uint32_t tn = t + sg.stride;
                     const bool more = tn < sg.end;
                     if (more) load_split_a<P, V, CG>(a, tn, own, oth, A);  // the neighbour vectors are dead
-                    if (update_item_h<P, V, true, false, AX>(sv, h, site0, rank0, c, a, J, K, ex, ey, ez, beta, acc)) {
+                    if (update_item_h<P, V, true, false, AX, CG>(sv, h, site0, rank0, c, a, J, K, ex, ey, ez, beta, acc,
+                                                                 oth, b0)) {
 #pragma unroll
                         for (int q = 0; q < 3; ++q) *reinterpret_cast<VT *>(own_w[q] + b0) = sv[q];
                     }
@@ -230,8 +232,9 @@ __device__ __forceinline__ void batch_pass(const BatchArgs &b, int s, int c) {
             for (uint32_t t = sg.begin + threadIdx.x; t < sg.end; t += sg.stride) {
                 StencilItem<P, V> it;
                 load_item<P, V, CG>(a, t, own, oth, it);
-                if (update_item<P, V, true, false, AX>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0,
-                                                       it.rank0, c, a, J, K, ex, ey, ez, beta, acc)) {
+                if (update_item<P, V, true, false, AX, CG>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p,
+                                                           it.site0, it.rank0, c, a, J, K, ex, ey, ez, beta, acc, oth,
+                                                           it.b0)) {
 #pragma unroll
                     for (int q = 0; q < 3; ++q) *reinterpret_cast<VT *>(own_w[q] + it.b0) = it.s[q];
                 }
@@ -404,7 +407,7 @@ __global__ void __launch_bounds__(kBlock, 2) batch_resident_kernel(const BatchAr
                 StencilItem<P, V> it;
                 load_item<P, V>(a, t, own, oth, it);
                 if (update_item<P, V, true, false, AX>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0,
-                                                       it.rank0, c, a, J, K, ex, ey, ez, beta, acc)) {
+                                                       it.rank0, c, a, J, K, ex, ey, ez, beta, acc, oth, it.b0)) {
 #pragma unroll
                     for (int q = 0; q < 3; ++q) *reinterpret_cast<VT *>(own_w[q] + it.b0) = it.s[q];
                 }

@@ -84,63 +84,116 @@ __device__ __forceinline__ void sphere_fp64(uint4 w, double &x, double &y, doubl
     y = r * sn;
 }
 
-// sin(pi t), cos(pi t) for t = m 2^-52 in [0, 2) (m < 2^53), by table lookup
-// and angle addition (Tang, "Table-lookup algorithms for elementary functions
-// and their error analysis", 1991): j = m 2^-42 rounded to the nearest
-// integer (0 .. 2048; j = 2048 is j = 0, the period being 2) and b = m - j 2^42
-// in [-2^41, 2^41), so t = j/1024 + b 2^-52 exactly.  sin, cos(pi j/1024) come
-// from a 2048-entry table (correctly rounded on the host); x = pi b 2^-52
-// (|x| <= pi 2^-11 < 0.00154) takes sin x = x - x^3/6 (first omitted term
-// below 7.2e-17) and cos x = 1 - c, c = x^2/2 - x^4/24 (first omitted below
-// 1.8e-20); then sin(a + x) = sin a + (cos a sin x - sin a c) and
-// cos(a + x) = cos a - (sin a sin x + cos a c).  Error below two units in the
-// last place, for 10 FP64 operations.
-constexpr double kPiTwoM52 = 3.141592653589793 * 0x1p-52;  // pi (FP64) 2^-52, exact scaling
-
-__device__ __forceinline__ void sincospi_tab(uint64_t m, const double2 *tab, double &sn, double &cs) {
-    const uint64_t j = (m + (1ull << 41)) >> 42;
-    const int64_t b = (int64_t)m - (int64_t)(j << 42);
-    const double x = (double)b * kPiTwoM52;
-    const double x2 = x * x;
-    const double sx = fma(x * x2, -1.0 / 6.0, x);
-    const double c = x2 * fma(x2, -1.0 / 24.0, 0.5);
-    const double2 t = __ldg(tab + (j & 2047u));
-    sn = fma(t.y, sx, fma(-t.x, c, t.x));
-    cs = fma(-t.x, sx, fma(-t.y, c, t.y));
+// ---- FP64 trial orientation in the integer pipe.  The FP64 pipe issues 2
+// instructions per cycle per SM, the integer units 32 (32x32->64 multiply) to
+// 128 (add, logic), so the sphere point is formed in 64-bit fixed point, about
+// 190 integer instructions, where FP64 took 26 that cost as much as 1600.
+// Every product keeps 61 bits or more below 1, so the results, rounded to
+// nearest, carry the error of that last rounding only.
+//
+// floor(a b / 2^64), low partial product left out: at most 3 too small.
+__device__ __forceinline__ uint64_t mulhi_64(uint64_t a, uint64_t b) {
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+    return (uint64_t)ah * bh + __umulhi(ah, bl) + __umulhi(al, bh);
 }
 
-// k 2^-s exactly, for an integer |k| < 2^53 and 0 < s <= 53: k converted
-// (exact), then s taken off its exponent field, which stays positive for
-// |k| >= 1; k = 0 gives +0.  Integer instructions in place of an FP64 multiply.
-__device__ __forceinline__ double scaled_int(int64_t k, int s) {
-    const double d = (double)k;
-    const double r = __hiloint2double(__double2hiint(d) - (s << 20), __double2loint(d));
-    return k == 0 ? 0.0 : r;
+// v 2^-s as a double rounded to nearest (e0 = 1085 - s), with the given sign.
+__device__ __forceinline__ double fixed_to_double(uint64_t v, int e0, bool neg) {
+    const int n = __clzll((long long)(v | 1ull));
+    const uint64_t w = v << n;  // leading bit at 63
+    const uint64_t mant = (w >> 11) + ((w >> 10) & 1ull);
+    const uint64_t bits = (mant + ((uint64_t)(uint32_t)(e0 - n) << 52)) | ((uint64_t)neg << 63);
+    return v == 0 ? 0.0 : __longlong_as_double((long long)bits);
 }
 
-// Trial orientation and acceptance uniform of one site, FP64 schedule
-// (Metropolis step (ii)); the sphere point of sphere_fp64 up to rounding:
-// 1 - z^2 is formed with one rounding (fma), and phi = pi v = pi t - pi
-// (t = v + 1) from the table: sin(pi v) = -sin(pi t), cos(pi v) = -cos(pi t).
-// uf is the acceptance uniform's top 24 bits: uf <= u < uf + 2^-24.
-__device__ __forceinline__ void draw_trial64(uint32_t site, uint32_t sweep, uint32_t colour, uint32_t replica,
-                                             uint32_t k0, uint32_t k1, const double2 *tab, double &tx, double &ty,
-                                             double &tz, double &u, float &uf) {
-    const uint32_t w2 = (kTagTrial << 24) | (colour << 8);
-    const uint4 a = philox10(make_uint4(site, sweep, w2, replica), k0, k1);
-    const uint4 b = philox10(make_uint4(site, sweep, w2 | 1u, replica), k0, k1);
-    const int64_t two52 = int64_t(1) << 52;
-    const int64_t iz = (int64_t)((((uint64_t)(a.x >> 5)) << 26) | (uint64_t)(a.y >> 6));
-    const uint64_t iv = (((uint64_t)(a.z >> 5)) << 26) | (uint64_t)(a.w >> 6);
-    tz = scaled_int(iz - two52, 52);
-    const double r = sqrt(fma(-tz, tz, 1.0));
-    double sn, cs;
-    sincospi_tab(iv, tab, sn, cs);
-    tx = -(r * cs);
-    ty = -(r * sn);
-    const uint64_t ip = (((uint64_t)(b.x >> 5)) << 26) | (uint64_t)(b.y >> 6);
-    u = scaled_int((int64_t)ip, 53);
-    uf = (float)(uint32_t)(ip >> 29) * 0x1p-24f;
+// The 53-bit uniform of two Philox words.
+__device__ __forceinline__ uint64_t bits53(uint32_t a, uint32_t b) {
+    return ((uint64_t)(a >> 5) << 26) | (uint64_t)(b >> 6);
+}
+
+// A trial spin and its components in FP32 (error below 2^-23).
+struct Trial64 {
+    double x, y, z;
+    float fx, fy, fz;
+};
+
+// The sphere point of sphere_fp64 from one Philox block.
+//  * z = (iz - 2^52) 2^-52 exactly.
+//  * r = sqrt((1 - |z|)(1 + |z|)): both factors are exact integers; 1 - |z| is
+//    scaled up by an even power of two, so their product W lies in
+//    [1/16, 1/2); sqrt(W) starts from the hardware reciprocal square root
+//    (2^-22) and takes two Newton steps on the exact residual, W - Y^2 (2^-44,
+//    then below 2^-60).
+//  * phi = pi v = pi t - pi, t = iv 2^-52: sin and cos of pi t by quadrant,
+//    table and angle addition (Tang, "Table-lookup algorithms for elementary
+//    functions and their error analysis", 1991): 2048 entries of sin, cos
+//    (pi j / 4096) in units of 2^-63, then theta < pi/2 2^-11 by
+//    sin theta = theta - theta^3/6 (first omitted term 2^-58.6) and
+//    1 - cos theta = theta^2/2 - theta^4/24 (omitted 2^-71).
+__device__ __forceinline__ Trial64 trial64(uint4 w, const ulonglong2 *tab) {
+    Trial64 t;
+    const uint64_t one = 1ull << 52;
+    const uint64_t iz = bits53(w.x, w.y), iv = bits53(w.z, w.w);
+    const bool zneg = iz < one;
+    const uint64_t m = zneg ? one - iz : iz - one;  // |z| 2^52
+    t.z = fixed_to_double(m, 1033, zneg);
+    t.fz = (float)(uint32_t)(m >> 21) * 0x1p-31f;
+    t.fz = zneg ? -t.fz : t.fz;
+
+    const uint64_t A = one - m;
+    const int sh = __clzll((long long)(A | 1ull)) & ~1;  // 10 .. 62
+    const uint64_t W = mulhi_64(A << sh, (one + m) << 10);
+    const float wf = (float)(uint32_t)(W >> 32) * 0x1p-32f;
+    const float rs = rsqrtf(fmaxf(wf, 0.0625f));
+    const uint32_t Y0 = __float2uint_rz(wf * rs * 0x1p32f);
+    const int32_t R = __float2int_rz(rs * 0x1p28f);  // (1 / (2 sqrt W)) 2^29
+    const int64_t E0 = (int64_t)(W - (uint64_t)Y0 * Y0);  // below 2^43
+    const int64_t d0 = (int64_t)(int32_t)(E0 >> 12) * R;  // units of 2^-81
+    const uint64_t Y1 = ((uint64_t)Y0 << 32) + (uint64_t)(d0 >> 17);
+    const int32_t E1 = (int32_t)(uint32_t)(W - mulhi_64(Y1, Y1));
+    const uint64_t Y2 = Y1 + (uint64_t)(((int64_t)E1 * R) >> 29);
+    const uint64_t r = Y2 >> ((sh >> 1) - 5);  // units of 2^-62
+
+    const uint32_t quad = (uint32_t)(iv >> 51);
+    const uint32_t j = (uint32_t)(iv >> 40) & 2047u;
+    const ulonglong2 sc = __ldg(tab + j);
+    const uint64_t u = mulhi_64(iv << 24, 0xC90FDAA22168C235ull);  // theta 2^11, units of 2^-63 (pi/2 2^63)
+    const uint64_t s2 = mulhi_64(u, u);                            // theta^2 2^22, units of 2^-62
+    const uint32_t s2h = (uint32_t)(s2 >> 32);
+    // (1 - cos theta) 2^23, units of 2^-62, and sin theta 2^11, units of 2^-63 (1/3 and 1/6 in 32 bits)
+    const uint64_t c = s2 - ((uint64_t)__umulhi(__umulhi(s2h, s2h), 0x55555555u) << 10);
+    const uint64_t sx = u - ((uint64_t)__umulhi(__umulhi(s2h, (uint32_t)(u >> 32)), 0x2AAAAAABu) << 12);
+    const uint64_t sn = sc.x + (mulhi_64(sc.y, sx) >> 10) - (mulhi_64(sc.x, c) >> 21);
+    const uint64_t cs = sc.y - (mulhi_64(sc.x, sx) >> 10) - (mulhi_64(sc.y, c) >> 21);
+    // x = -r cos(pi t), y = -r sin(pi t)
+    const bool odd = quad & 1u;
+    const uint64_t X = mulhi_64(r, odd ? sn : cs), Y = mulhi_64(r, odd ? cs : sn);  // units of 2^-61
+    const bool xneg = quad == 0u || quad == 3u, yneg = quad < 2u;
+    t.x = fixed_to_double(X, 1024, xneg);
+    t.y = fixed_to_double(Y, 1024, yneg);
+    t.fx = (float)(uint32_t)(X >> 32) * 0x1p-29f;
+    t.fy = (float)(uint32_t)(Y >> 32) * 0x1p-29f;
+    t.fx = xneg ? -t.fx : t.fx;
+    t.fy = yneg ? -t.fy : t.fy;
+    return t;
+}
+
+// The Philox blocks of one site's FP64 trial: call 0 the orientation, call 1 the acceptance uniform.
+__device__ __forceinline__ uint4 trial64_block(uint32_t site, uint32_t sweep, uint32_t colour, uint32_t call,
+                                               uint32_t replica, uint32_t k0, uint32_t k1) {
+    return philox10(make_uint4(site, sweep, (kTagTrial << 24) | (colour << 8) | call, replica), k0, k1);
+}
+
+// A double's value truncated to a float by its bit fields (the conversion
+// instruction runs at the FP64 pipe's rate): within 2^-23 of its size for
+// 2^-126 <= |v| < 2^128, smaller ones come out below 2^-125.  big collects the
+// high word of the largest |v| seen, by which the caller knows the range held.
+__device__ __forceinline__ float narrow(double v, int &big) {
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    const int u = hi & 0x7FFFFFFF;
+    big = max(big, u);
+    const uint32_t f = __funnelshift_l((uint32_t)lo, (uint32_t)max(u - 0x38000000, 0), 3);
+    return __uint_as_float((f & 0x7FFFFFFFu) | ((uint32_t)hi & 0x80000000u));
 }
 
 // ---- FP32 arithmetic of one site (float) or of the two sites of a Philox
@@ -346,6 +399,19 @@ __device__ __forceinline__ bool accept64(double x, double u, float uf) {
         if (uf > __fmul_rn(e, 1.0f + 3e-5f)) return false;
     }
     return u <= exp(x);
+}
+
+// The FP64 decision from FP32 values of the spins and the field: x = -beta dH
+// is off by at most a.fdelta (PassArgs), beside 2.4e-5 |x| / 80 from five FP32
+// roundings and 2^-22 from the hardware 2^x, which the factors 1 -+ 4e-5 cover
+// for |x| <= 80; below, P <= e^x < 2^-115 is decided by P's top 24 bits alone,
+// and dH <= 0 (e^x >= 1 > P) is the same rule.  1 accepted, 0 rejected, -1
+// within the bounds of each other: FP64 decides (in about 1 site of 10^5).
+__device__ __forceinline__ int decide64(float x, float delta, float uf) {
+    const float lo = ex2_hw(__fmul_rn(x - delta, 1.44269504088896341f));
+    const float hi = ex2_hw(__fmul_rn(x + delta, 1.44269504088896341f));
+    if (__fadd_rn(uf, 0x1p-24f) < __fmul_rn(lo, 1.0f - 4e-5f)) return 1;
+    return uf > __fmul_rn(hi, 1.0f + 4e-5f) ? 0 : -1;
 }
 
 // ZAX: the easy axis is e = (0, 0, 1) exactly, so S.e = S_z (what the three
@@ -615,6 +681,7 @@ __device__ __forceinline__ float neg_beta_log2e(float beta) { return f_mul(-beta
 // picks (xh-1, xh) or (xh, xh+1) for the x neighbours) and its rows at y-1,
 // y+1, z-1, z+1.  FP32 / FP16 add two sites at a time as the lanes of float2
 // (identical per lane to the scalar adds).
+// FP32 / FP16 here; FP64 in item_fields64.
 template <int P, int V>
 __device__ __forceinline__ void item_fields(const Vec<typename Tr<P>::S, V> (&o)[3],
                                             const Vec<typename Tr<P>::S, V> (&nym)[3],
@@ -625,15 +692,7 @@ __device__ __forceinline__ void item_fields(const Vec<typename Tr<P>::S, V> (&o)
     using C = typename Tr<P>::C;
     auto xm_of = [&](int k, int q) -> C { return p ? to_c(o[q].v[k]) : (k == 0 ? ed[q] : to_c(o[q].v[k - 1])); };
     auto xp_of = [&](int k, int q) -> C { return p ? (k == V - 1 ? ed[q] : to_c(o[q].v[k + 1])) : to_c(o[q].v[k]); };
-    if constexpr (P == HS_FP64) {
-#pragma unroll
-        for (int k = 0; k < V; ++k)
-#pragma unroll
-            for (int q = 0; q < 3; ++q)
-                h[q][k] = ((((xm_of(k, q) + xp_of(k, q)) + to_c(nym[q].v[k])) + to_c(nyp[q].v[k])) +
-                           to_c(nzm[q].v[k])) +
-                          to_c(nzp[q].v[k]);
-    } else if constexpr (P == HS_FP16) {
+    if constexpr (P == HS_FP16) {
         // binary16 operands added straight into the FP32 sum (add_half: one
         // rounding per add, the same sums as widening each operand first)
 #pragma unroll
@@ -676,40 +735,153 @@ __device__ __forceinline__ void item_fields(const Vec<typename Tr<P>::S, V> (&o)
     }
 }
 
+// FP64: the field the decision needs in FP32 (f), and where the energy needs
+// it (wide: the later colour's fused measurement, or the tensor term) in FP64
+// (d), its FP32 form taken from that.  The 15 FP64 additions a site cost as
+// much issue time of their pipe as 480 integer instructions, so the narrow
+// form converts every operand by its bit fields instead.  ok: every component
+// the FP32 form was made from has a size of at most 1 + 2^-12 (unit vectors),
+// which fdelta's error bound rests on.
+template <int V>
+struct Field64 {
+    double d[3][V];
+    float f[3][V];
+    bool ok;
+};
+
+template <int V>
+__device__ __forceinline__ void item_fields64(const Vec<double, V> (&o)[3], const Vec<double, V> (&nym)[3],
+                                              const Vec<double, V> (&nyp)[3], const Vec<double, V> (&nzm)[3],
+                                              const Vec<double, V> (&nzp)[3], const double (&ed)[3], uint32_t p,
+                                              bool wide, Field64<V> &F) {
+    int big = 0;
+    if (wide) {
+#pragma unroll
+        for (int k = 0; k < V; ++k)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const double xm = p ? o[q].v[k] : (k == 0 ? ed[q] : o[q].v[k == 0 ? 0 : k - 1]);
+                const double xp = p ? (k == V - 1 ? ed[q] : o[q].v[k == V - 1 ? 0 : k + 1]) : o[q].v[k];
+                F.d[q][k] = ((((xm + xp) + nym[q].v[k]) + nyp[q].v[k]) + nzm[q].v[k]) + nzp[q].v[k];
+                F.f[q][k] = narrow(F.d[q][k], big);
+            }
+        F.ok = big <= 0x40190000;  // 6.25
+    } else {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            float x[V];  // the other colour's same row
+#pragma unroll
+            for (int k = 0; k < V; ++k) x[k] = narrow(o[q].v[k], big);
+            const float e = narrow(ed[q], big);
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+                // p: x neighbours (k, k + 1), else (k - 1, k); beyond the row's end the edge element
+                const float other = p ? (k == V - 1 ? e : x[k == V - 1 ? 0 : k + 1]) : (k == 0 ? e : x[k == 0 ? 0 : k - 1]);
+                float h = f_add(x[k], other);
+                h = f_add(h, narrow(nym[q].v[k], big));
+                h = f_add(h, narrow(nyp[q].v[k], big));
+                h = f_add(h, narrow(nzm[q].v[k], big));
+                F.f[q][k] = f_add(h, narrow(nzp[q].v[k], big));
+            }
+        }
+        F.ok = big <= 0x3FF00100;  // 1 + 2^-12
+    }
+}
+
+// Where a work item's operands lie, for the few sites whose FP32 decision is
+// open: the other colour's planes and the item's first element.
+struct ItemSource {
+    const double *o[3];
+    uint32_t b0;
+};
+
+// One component of a site's FP64 field, read again from the other colour's
+// plane o (which no pass of this colour writes); b = the site's element.
+template <bool CG>
+__device__ __noinline__ double stencil_field64(const double *o, uint32_t b, uint32_t Lh, uint32_t Ly, uint32_t Lz,
+                                               uint32_t par) {
+    const uint32_t row = b / Lh, x = b - row * Lh, z = row / Ly, y = row - z * Ly;
+    const uint32_t p = (y + z + par) & 1u;
+    auto at = [&](uint32_t zz, uint32_t yy, uint32_t xx) {
+        const double *q = o + ((size_t)zz * Ly + yy) * Lh + xx;
+        if constexpr (CG)
+            return __ldcg(q);
+        else
+            return *q;
+    };
+    double h = at(z, y, p ? x : (x == 0 ? Lh - 1 : x - 1));
+    h += at(z, y, p ? (x == Lh - 1 ? 0 : x + 1) : x);
+    h += at(z, y == 0 ? Ly - 1 : y - 1, x);
+    h += at(z, y == Ly - 1 ? 0 : y + 1, x);
+    h += at(z == 0 ? Lz - 1 : z - 1, y, x);
+    h += at(z == Lz - 1 ? 0 : z + 1, y, x);
+    return h;
+}
+
+// The plain FP64 rule, for a decision that FP32 left open.
+template <bool ZAX>
+__device__ __noinline__ bool accept_wide(double sx, double sy, double sz, double tx, double ty, double tz, double hx,
+                                         double hy, double hz, double J, double K, double ex, double ey, double ez,
+                                         double beta, double u, float uf) {
+    return metropolis<double, false, ZAX>(sx, sy, sz, tx, ty, tz, hx, hy, hz, J, K, ex, ey, ez, beta, u, uf).acc;
+}
+
 // Metropolis steps (ii)-(iii) for the V sites of one FP64 work item (see
-// update_item_h); ZAX as in metropolis.
-template <int V, bool MEAS, bool TEN, bool ZAX>
-__device__ __forceinline__ bool update_fp64(Vec<double, V> (&s)[3], const double (&h)[3][V], uint32_t site0, int c,
+// update_item_h); ZAX as in metropolis.  Spins, trials and sums are FP64; the
+// decision is the FP64 rule's, taken from FP32 values wherever their error
+// bound settles it (decide64).
+template <int V, bool MEAS, bool TEN, bool ZAX, bool CG>
+__device__ __forceinline__ bool update_fp64(Vec<double, V> (&s)[3], const Field64<V> &F, uint32_t site0, int c,
                                             const PassArgs &a, double J, double K, double ex, double ey, double ez,
-                                            double beta, SiteAcc<HS_FP64> &acc) {
-    using C = double;
+                                            double beta, SiteAcc<HS_FP64> &acc, const ItemSource &src) {
     bool any = false;
 #pragma unroll
     for (int k = 0; k < V; ++k) {
-        C tx, ty, tz, u;
-        float uf;
-        draw_trial64(site0 + 2u * k, a.sweep, (uint32_t)c, a.replica, a.key0, a.key1, a.sc_tab, tx, ty, tz, u,
-                     uf);
-        C sx = s[0].v[k], sy = s[1].v[k], sz = s[2].v[k];
-        const SiteDots<C> d = metropolis<C, TEN, ZAX>(sx, sy, sz, tx, ty, tz, h[0][k], h[1][k], h[2][k], J, K,
-                                                      ex, ey, ez, beta, u, uf, a.A);
-        if (d.acc) {
-            sx = tx;
-            sy = ty;
-            sz = tz;
-            s[0].v[k] = tx;
-            s[1].v[k] = ty;
-            s[2].v[k] = tz;
+        const uint32_t site = site0 + 2u * k;
+        const Trial64 t =
+            trial64(trial64_block(site, a.sweep, (uint32_t)c, 0u, a.replica, a.key0, a.key1), a.sc_tab);
+        const uint4 pw = trial64_block(site, a.sweep, (uint32_t)c, 1u, a.replica, a.key0, a.key1);
+        const float uf = (float)(pw.x >> 8) * 0x1p-24f;  // P's top 24 bits
+        double sx = s[0].v[k], sy = s[1].v[k], sz = s[2].v[k];
+        bool ac;
+        if constexpr (TEN) {
+            const double u = (double)bits53(pw.x, pw.y) * 0x1p-53;
+            ac = metropolis<double, true, ZAX>(sx, sy, sz, t.x, t.y, t.z, F.d[0][k], F.d[1][k], F.d[2][k], J, K, ex, ey,
+                                               ez, beta, u, uf, a.A)
+                     .acc;
+        } else {
+            int big = 0;
+            const float fx = narrow(sx, big), fy = narrow(sy, big), fz = narrow(sz, big);
+            const Dots32<float> d =
+                site_math32<float, false, ZAX>(fx, fy, fz, t.fx, t.fy, t.fz, F.f[0][k], F.f[1][k], F.f[2][k], a.fJ,
+                                               a.fK, a.fe[0], a.fe[1], a.fe[2]);
+            int dec = decide64(-a.fbeta * d.dH, a.fdelta, uf);
+            if (!F.ok || big > 0x3FF00100) dec = -1;
+            if (dec < 0) {
+                double h[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    h[q] = stencil_field64<CG>(src.o[q], src.b0 + k, (uint32_t)a.Lh, (uint32_t)a.Ly, (uint32_t)a.Lz,
+                                               (uint32_t)(a.colour + a.zpar));
+                dec = accept_wide<ZAX>(sx, sy, sz, t.x, t.y, t.z, h[0], h[1], h[2], J, K, ex, ey, ez, beta,
+                                       (double)bits53(pw.x, pw.y) * 0x1p-53, uf);
+            }
+            ac = dec > 0;
+        }
+        if (ac) {
+            s[0].v[k] = sx = t.x;
+            s[1].v[k] = sy = t.y;
+            s[2].v[k] = sz = t.z;
             any = true;
             ++acc.n;
         }
         if (MEAS) {
             // bond energy counted at the later colour's end: pass 1 owns
             // every sc bond, pass 0 only the anisotropy term
-            const C e_new = d.acc ? d.pe : d.se;
-            acc.k = fma(e_new, e_new, acc.k);
-            if (TEN) acc.e -= d.acc ? d.qt : d.qs;
-            if (c == 1) acc.j += d.acc ? d.th : d.sh;
+            const double se = ZAX ? sz : sx * ex + sy * ey + sz * ez;
+            acc.k = fma(se, se, acc.k);
+            if (TEN) acc.e -= quad64(sx, sy, sz, a.A);
+            if (c == 1) acc.j = fma(sz, F.d[2][k], fma(sy, F.d[1][k], fma(sx, F.d[0][k], acc.j)));
             acc.x += sx;
             acc.y += sy;
             acc.z += sz;
@@ -818,23 +990,50 @@ __device__ __forceinline__ bool update_f32(Vec<typename Tr<P>::S, V> (&s)[3], co
     return any;
 }
 
+// A work item's local fields as its precision keeps them.
+template <int P, int V>
+struct ItemField {
+    using T = typename Tr<P>::C[3][V];
+};
+template <int V>
+struct ItemField<HS_FP64, V> {
+    using T = Field64<V>;
+};
+
+// Step (i) of a work item from its raw operands.
+template <int P, int V, bool MEAS, bool TEN>
+__device__ __forceinline__ void fields_of(const Vec<typename Tr<P>::S, V> (&o)[3],
+                                          const Vec<typename Tr<P>::S, V> (&nym)[3],
+                                          const Vec<typename Tr<P>::S, V> (&nyp)[3],
+                                          const Vec<typename Tr<P>::S, V> (&nzm)[3],
+                                          const Vec<typename Tr<P>::S, V> (&nzp)[3], const typename Tr<P>::C (&ed)[3],
+                                          uint32_t p, int c, typename ItemField<P, V>::T &h) {
+    if constexpr (P == HS_FP64)
+        item_fields64<V>(o, nym, nyp, nzm, nzp, ed, p, TEN || (MEAS && c == 1), h);
+    else
+        item_fields<P, V>(o, nym, nyp, nzm, nzp, ed, p, h);
+}
+
 // AX = 1: the kernel was chosen for e = (0, 0, 1) at launch, so S.e = S_z
 // with no branch (the FP32 register stencil's form); AX = 2: the same with
 // K = +0 (the FP32 and FP16 batch kernels); AX = 0: FP64 and FP16 decide per
 // work item from PassArgs::zaxis, FP32 takes the general products.
-template <int P, int V, bool MEAS, bool TEN = false, int AX = 0>
-__device__ __forceinline__ bool update_item_h(Vec<typename Tr<P>::S, V> (&s)[3], const typename Tr<P>::C (&h)[3][V],
-                                              uint32_t site0, uint32_t rank0, int c, const PassArgs &a,
-                                              typename Tr<P>::C J, typename Tr<P>::C K, typename Tr<P>::C ex,
-                                              typename Tr<P>::C ey, typename Tr<P>::C ez, typename Tr<P>::C beta,
-                                              SiteAcc<P> &acc) {
+// oth, b0: where the item's neighbours lie (FP64; CG as in ld_val).
+template <int P, int V, bool MEAS, bool TEN = false, int AX = 0, bool CG = false>
+__device__ __forceinline__ bool update_item_h(Vec<typename Tr<P>::S, V> (&s)[3],
+                                              const typename ItemField<P, V>::T &h, uint32_t site0, uint32_t rank0,
+                                              int c, const PassArgs &a, typename Tr<P>::C J, typename Tr<P>::C K,
+                                              typename Tr<P>::C ex, typename Tr<P>::C ey, typename Tr<P>::C ez,
+                                              typename Tr<P>::C beta, SiteAcc<P> &acc,
+                                              const typename Tr<P>::S *const (&oth)[3], uint32_t b0) {
     if constexpr (P == HS_FP64) {
         // one uniform branch per work item: the item body with S.e = S_z
-        // (e = (0, 0, 1), the FP64 pipe spared six operations per site) or
-        // with the general dot products
+        // (e = (0, 0, 1)) or with the general dot products
+        const ItemSource src{{oth[0], oth[1], oth[2]}, b0};
         if constexpr (!TEN)
-            if (a.zaxis) return update_fp64<V, MEAS, false, true>(s, h, site0, c, a, J, K, ex, ey, ez, beta, acc);
-        return update_fp64<V, MEAS, TEN, false>(s, h, site0, c, a, J, K, ex, ey, ez, beta, acc);
+            if (a.zaxis)
+                return update_fp64<V, MEAS, false, true, CG>(s, h, site0, c, a, J, K, ex, ey, ez, beta, acc, src);
+        return update_fp64<V, MEAS, TEN, false, CG>(s, h, site0, c, a, J, K, ex, ey, ez, beta, acc, src);
     } else {
         if constexpr (AX >= 1 && !TEN)
             return update_f32<P, V, MEAS, false, true, AX == 2>(s, h, rank0, c, a, J, K, ex, ey, ez, beta, acc);
@@ -850,7 +1049,7 @@ __device__ __forceinline__ bool update_item_h(Vec<typename Tr<P>::S, V> (&s)[3],
 }
 
 // The same from the raw operands: step (i) then steps (ii)-(iii).
-template <int P, int V, bool MEAS, bool TEN = false, int AX = 0>
+template <int P, int V, bool MEAS, bool TEN = false, int AX = 0, bool CG = false>
 __device__ __forceinline__ bool update_item(Vec<typename Tr<P>::S, V> (&s)[3], const Vec<typename Tr<P>::S, V> (&o)[3],
                                             const Vec<typename Tr<P>::S, V> (&nym)[3],
                                             const Vec<typename Tr<P>::S, V> (&nyp)[3],
@@ -859,10 +1058,10 @@ __device__ __forceinline__ bool update_item(Vec<typename Tr<P>::S, V> (&s)[3], c
                                             uint32_t p, uint32_t site0, uint32_t rank0, int c, const PassArgs &a,
                                             typename Tr<P>::C J, typename Tr<P>::C K, typename Tr<P>::C ex,
                                             typename Tr<P>::C ey, typename Tr<P>::C ez, typename Tr<P>::C beta,
-                                            SiteAcc<P> &acc) {
-    typename Tr<P>::C h[3][V];
-    item_fields<P, V>(o, nym, nyp, nzm, nzp, ed, p, h);
-    return update_item_h<P, V, MEAS, TEN, AX>(s, h, site0, rank0, c, a, J, K, ex, ey, ez, beta, acc);
+                                            SiteAcc<P> &acc, const typename Tr<P>::S *const (&oth)[3], uint32_t b0) {
+    typename ItemField<P, V>::T h;
+    fields_of<P, V, MEAS, TEN>(o, nym, nyp, nzm, nzp, ed, p, c, h);
+    return update_item_h<P, V, MEAS, TEN, AX, CG>(s, h, site0, rank0, c, a, J, K, ex, ey, ez, beta, acc, oth, b0);
 }
 
 // Vector load, optionally L2-only (ld.global.cg).  A kernel that reads data

@@ -94,7 +94,8 @@ struct PassArgs {
     int tensor;             // 1: the on-site anisotropy tensor term is on
     double A[6];            // its symmetric tensor (xx, yy, zz, xy, xz, yz)
     float fA[6];
-    const double2 *sc_tab;  // FP64 trial: sin, cos(pi j / 1024), j = 0..2047
+    const ulonglong2 *sc_tab;  // FP64 trial: sin, cos(pi j / 4096) in units of 2^-63, j = 0..2047
+    float fdelta;           // FP64: bound on the error of the FP32 form of beta dH (decision_band)
     int zaxis;              // 1: e = (0, 0, 1) exactly (the FP64 stencil takes S.e = S_z)
     uint32_t key0, key1, replica, sweep;
     double *partials;       // [ring slots][n_colours][n_blocks][kPartials]; a slab has kSlabSets sets per colour
@@ -140,6 +141,25 @@ struct Layout {
     int64_t n_pad;
     int64_t colour_begin[65];  // renumbered colour ranges (n_colours + 1 entries)
 };
+
+// How far the FP32 form of beta dH may be from the FP64 one, for spins whose
+// components are at most 1 + 2^-12 and six neighbours at most.  In units of
+// 2^-24, per field component: six operands truncated to FP32 (2 each) and five
+// additions of sums up to 6 (6 each), 42; so S.h is off by at most
+// sqrt(3) 42 + 2 6 (S truncated) + 3 6 (the product's roundings) = 103, S'.h by
+// less, and J (S.h - S'.h) by 2 103 + 12 + 2 12 = 242 < 2e-5 / 2^-24 = 335; a
+// field taken from FP64 is closer.  Up to twelve neighbours (the table's fcc):
+// fields up to 12, eleven additions, twice and a half the bound.  The
+// uniaxial term: S.e off by 12 each, times the sum of at most 2: 60 < 1e-5 /
+// 2^-24 = 167.  Infinite (FP64 decides every site) where J, K or beta leave
+// FP32's range.
+inline float decision_band(double beta, double J, double K, int width) {
+    auto fits = [](double v) { return v == 0.0 || (v >= 1e-30 && v <= 1e30); };
+    const double aJ = J < 0 ? -J : J, aK = K < 0 ? -K : K;
+    if (!fits(beta) || !fits(aJ) || !fits(aK) || !fits(beta * aJ) || !fits(beta * aK) || width > 12)
+        return __builtin_inff();
+    return (float)(beta * (aJ * (width > 6 ? 6e-5 : 2e-5) + aK * 1e-5) * 1.001);
+}
 
 size_t storage_size(int precision);
 

@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kBlock, 2) sc_pass_kernel(const PassArgs a) {
     const uint32_t stride = gridDim.x * blockDim.x;
     auto compute = [&](StencilItem<P, V> &it) {
         if (update_item<P, V, MEAS, TEN, AX>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0, it.rank0,
-                                             c, a, J, K, ex, ey, ez, beta, acc)) {
+                                             c, a, J, K, ex, ey, ez, beta, acc, oth, it.b0)) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) *reinterpret_cast<VT *>(own_w[q] + it.b0) = it.s[q];
         }
@@ -91,14 +91,15 @@ __global__ void __launch_bounds__(kBlock, 2) sc_pass_kernel(const PassArgs a) {
             while (true) {
                 VT nym[3], nyp[3];
                 load_split_b<P, V>(A, oth, nym, nyp);
-                C h[3][V];
-                item_fields<P, V>(A.o, nym, nyp, A.nzm, A.nzp, A.ed, A.f.p, h);
+                typename ItemField<P, V>::T h;
+                fields_of<P, V, MEAS, TEN>(A.o, nym, nyp, A.nzm, A.nzp, A.ed, A.f.p, c, h);
                 VT sv[3] = {A.s[0], A.s[1], A.s[2]};
                 const uint32_t b0 = A.f.b0, site0 = A.f.site0, rank0 = A.f.rank0;
                 const uint32_t tn = t + stride;
                 const bool more = tn < n_items;
                 if (more) load_split_a<P, V, false, DIR>(a, tn, own, oth, A);  // the neighbour vectors are dead now
-                if (update_item_h<P, V, MEAS, TEN, AX>(sv, h, site0, rank0, c, a, J, K, ex, ey, ez, beta, acc)) {
+                if (update_item_h<P, V, MEAS, TEN, AX>(sv, h, site0, rank0, c, a, J, K, ex, ey, ez, beta, acc, oth,
+                                                       b0)) {
 #pragma unroll
                     for (int q = 0; q < 3; ++q) *reinterpret_cast<VT *>(own_w[q] + b0) = sv[q];
                 }
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(kBlock, 2) sc_pipe_kernel(const PassArgs a) {
             const bool more = tn < n_items;
             if (more) f = pipe_issue<P, V>(a, tn, own, oth, slot_v, slot_e);
             if (update_item<P, V, MEAS, false, AX>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0,
-                                                   it.rank0, c, a, J, K, ex, ey, ez, beta, acc)) {
+                                                   it.rank0, c, a, J, K, ex, ey, ez, beta, acc, oth, it.b0)) {
 #pragma unroll
                 for (int q = 0; q < 3; ++q) *reinterpret_cast<VT *>(own_w[q] + it.b0) = it.s[q];
             }
@@ -326,13 +327,27 @@ __global__ void __launch_bounds__(kBlock, 2) sc_march_kernel(const PassArgs a) {
             StencilItem<P, V> item;
             load_item_at<P, V>(a, y0 + yl, z, xv, own, oth, item);
             if (update_item<P, V, MEAS>(item.s, item.o, item.nym, item.nyp, item.nzm, item.nzp, item.ed, item.p,
-                                        item.site0, item.rank0, c, a, J, K, ex, ey, ez, beta, acc)) {
+                                        item.site0, item.rank0, c, a, J, K, ex, ey, ez, beta, acc, oth,
+                                        item.b0)) {
 #pragma unroll
                 for (int k = 0; k < 3; ++k) *reinterpret_cast<VT *>(own_w[k] + item.b0) = item.s[k];
             }
         }
     }
     write_partials<C, MEAS>(a, acc.E(J, K), acc.X(), acc.Y(), acc.Z(), acc.n);
+}
+
+// A site's FP64 field, its neighbours read again through the table (for a decision that FP32 left open).
+__device__ __noinline__ double3 table_field64(const Vec<double, 4> *spins, const int32_t *nbr, int64_t i, int64_t n_pad,
+                                              int width) {
+    double3 h = make_double3(0.0, 0.0, 0.0);
+    for (int k = 0; k < width; ++k) {
+        const Vec<double, 4> n = spins[__ldg(nbr + (int64_t)k * n_pad + i)];
+        h.x += n.v[0];
+        h.y += n.v[1];
+        h.z += n.v[2];
+    }
+    return h;
 }
 
 // ----------------------------------------------------------------- table pass
@@ -371,11 +386,32 @@ __global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (W > 0 ? 4 : 5)) ta
     for (int64_t i = a.begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.end; i += stride) {
         C hx = C(0), hy = C(0), hz = C(0);
         C lx = C(0), ly = C(0), lz = C(0);
+        // FP64 without the tensor: the field in FP32 (the decision's), the energy's part of it in FP64
+        constexpr bool kNarrow = P == HS_FP64 && !TEN;
+        float gx = 0.0f, gy = 0.0f, gz = 0.0f;
+        int big = 0;
         if (PFL2 && i + stride < a.end) {
             for (int k = 0; k < a.width; ++k)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(a.nbr + (int64_t)k * a.n_pad + i + stride));
             asm volatile("prefetch.global.L2 [%0];" ::"l"(spins + i + stride));
         }
+        auto add = [&](int32_t j, const S4 &n) {
+            const C nx = to_c(n.v[0]), ny = to_c(n.v[1]), nz = to_c(n.v[2]);
+            if constexpr (kNarrow) {
+                gx = f_add(gx, narrow(nx, big));
+                gy = f_add(gy, narrow(ny, big));
+                gz = f_add(gz, narrow(nz, big));
+            } else {
+                hx += nx;
+                hy += ny;
+                hz += nz;
+            }
+            if (MEAS && j < a.colour_begin) {
+                lx += nx;
+                ly += ny;
+                lz += nz;
+            }
+        };
         if constexpr (W > 0) {
             int32_t jj[W];
             S4 nn[W];
@@ -384,42 +420,45 @@ __global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (W > 0 ? 4 : 5)) ta
 #pragma unroll
             for (int k = 0; k < W; ++k) nn[k] = spins[jj[k]];
 #pragma unroll
-            for (int k = 0; k < W; ++k) {
-                const C nx = to_c(nn[k].v[0]), ny = to_c(nn[k].v[1]), nz = to_c(nn[k].v[2]);
-                hx += nx;
-                hy += ny;
-                hz += nz;
-                if (MEAS && jj[k] < a.colour_begin) {
-                    lx += nx;
-                    ly += ny;
-                    lz += nz;
-                }
-            }
+            for (int k = 0; k < W; ++k) add(jj[k], nn[k]);
         } else {
             for (int k = 0; k < a.width; ++k) {
                 const int32_t j = __ldg(a.nbr + (int64_t)k * a.n_pad + i);
-                const S4 n = spins[j];
-                const C nx = to_c(n.v[0]), ny = to_c(n.v[1]), nz = to_c(n.v[2]);
-                hx += nx;
-                hy += ny;
-                hz += nz;
-                if (MEAS && j < a.colour_begin) {
-                    lx += nx;
-                    ly += ny;
-                    lz += nz;
-                }
+                add(j, spins[j]);
             }
         }
         S4 s = spins[i];
         C sx = to_c(s.v[0]), sy = to_c(s.v[1]), sz = to_c(s.v[2]);
-        C tx, ty, tz, u;
+        C tx, ty, tz;
         bool accepted;
         if constexpr (P == HS_FP64) {
-            float uf;
-            draw_trial64(__ldg(a.nat + i), a.sweep, (uint32_t)a.colour, a.replica, a.key0, a.key1, a.sc_tab, tx, ty,
-                         tz, u, uf);
-            accepted = metropolis<C, TEN>(sx, sy, sz, tx, ty, tz, hx, hy, hz, J, K, ex, ey, ez, beta, u, uf, a.A).acc;
+            const uint32_t site = __ldg(a.nat + i);
+            const Trial64 t =
+                trial64(trial64_block(site, a.sweep, (uint32_t)a.colour, 0u, a.replica, a.key0, a.key1), a.sc_tab);
+            const uint4 pw = trial64_block(site, a.sweep, (uint32_t)a.colour, 1u, a.replica, a.key0, a.key1);
+            const float uf = (float)(pw.x >> 8) * 0x1p-24f;
+            tx = t.x;
+            ty = t.y;
+            tz = t.z;
+            if constexpr (kNarrow) {
+                const float fx = narrow(sx, big), fy = narrow(sy, big), fz = narrow(sz, big);
+                const Dots32<float> d = site_math32<float>(fx, fy, fz, t.fx, t.fy, t.fz, gx, gy, gz, a.fJ, a.fK,
+                                                           a.fe[0], a.fe[1], a.fe[2]);
+                int dec = decide64(-a.fbeta * d.dH, a.fdelta, uf);
+                if (big > 0x3FF00100) dec = -1;  // 1 + 2^-12: no unit vectors
+                if (dec < 0) {
+                    const double3 h = table_field64(spins, a.nbr, i, a.n_pad, a.width);
+                    dec = accept_wide<false>(sx, sy, sz, tx, ty, tz, h.x, h.y, h.z, J, K, ex, ey, ez, beta,
+                                             (double)bits53(pw.x, pw.y) * 0x1p-53, uf);
+                }
+                accepted = dec > 0;
+            } else {
+                accepted = metropolis<C, TEN>(sx, sy, sz, tx, ty, tz, hx, hy, hz, J, K, ex, ey, ez, beta,
+                                              (double)bits53(pw.x, pw.y) * 0x1p-53, uf, a.A)
+                               .acc;
+            }
         } else {
+            float u;
             draw_trial_rank<P>((uint32_t)(i - a.colour_begin), a.sweep, (uint32_t)a.colour, a.replica, a.key0,
                                a.key1, tx, ty, tz, u);
             const Dots32<float> d =
@@ -566,12 +605,12 @@ __global__ void __launch_bounds__(kBlock) sc_measure_kernel(const PassArgs a, co
         for (uint64_t t = t0; t < n_items; t += stride) {
             StencilItem<P, V> it;
             load((uint32_t)t, it);
-            double h[3][V];
-            item_fields<P, V>(it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, h);
+            Field64<V> h;
+            item_fields64<V>(it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, true, h);
 #pragma unroll
             for (int j = 0; j < V; ++j)
 #pragma unroll
-                for (int q = 0; q < 3; ++q) b = fma(it.s[q].v[j], h[q][j], b);
+                for (int q = 0; q < 3; ++q) b = fma(it.s[q].v[j], h.d[q][j], b);
             own(it.s);
         }
         write_partials<double, true>(a, -a.J * b - (GEN ? accG : (a.K == 0.0 ? 0.0 : a.K * k)), m[0], m[1], m[2], 0u);
