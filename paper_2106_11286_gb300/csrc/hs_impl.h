@@ -178,7 +178,7 @@ cudaError_t launch_gather(int precision, const Layout &L, double *d_xyz, cudaStr
 cudaError_t launch_measure(int precision, const Layout &L, const PassArgs &a, int n_blocks, cudaStream_t s);
 int measure_blocks(const Layout &L, int n_sm, int max_blocks);
 // Fold ring slots 0 .. n_slots-1 (sweeps of a.n_colours passes each, in sweep
-// order) into the accumulator: one CTA per slot sums it, then one thread
+// order) into the accumulator: one CTA per slot sums it, the last of them
 // applies the totals in order.  1 <= n_slots <= kRingMax.
 cudaError_t launch_fold(const PassArgs &a, int n_slots, cudaStream_t s);
 int pass_blocks(int precision, const Layout &L, int n_sm, int blocks_per_sm);

@@ -15,8 +15,8 @@
 // per CTA and pass, in a ring of slot sets, one per sweep of a group of up to
 // 64.  Within hs_sweep the passes only write slots; after each full group
 // (and after the loop) a ring fold sums every sweep's slots in a fixed order
-// (bit-reproducible), one CTA per sweep, and one thread applies the totals to
-// the FP64 accumulator in sweep order, so no pass carries a serial reduction
+// (bit-reproducible), one CTA per sweep, and the last of them applies the
+// totals to the FP64 accumulator in sweep order, so no pass carries a serial reduction
 // (a last-arriving CTA reducing inside the finishing pass cost 8 % at 256^3,
 // a fold in the next sweep's first pass 5 %).  Single passes and standalone
 // measurements keep the last-arriving-CTA form.
@@ -760,8 +760,51 @@ __global__ void __launch_bounds__(kBlock) table_measure_kernel(const PassArgs a,
 // ----------------------------------------------------------------- fold
 // Ring fold, after the last pass of a group of sweeps: CTA i sums ring slot i
 // (sweep i of the group) and writes that sweep's record (its totals and
-// observables) ...
-__global__ void __launch_bounds__(kBlock) fold_sum_kernel(const PassArgs a) {
+// observables); the last CTA to finish adds the records to the accumulator in
+// sweep order, one lane per accumulated quantity.  Bound by that serial chain
+// of FP64 additions, one per sweep and quantity: 64 of them in parallel lanes
+// over records staged in shared memory, where one thread walking all of them
+// through global memory took 26 us for 50 sweeps, in a launch of its own.
+__device__ void fold_apply(const PassArgs &a, int n_slots) {
+    __shared__ double s_rec[kRingMax][kSweepRecord];
+    for (int k = threadIdx.x; k < n_slots * kSweepRecord; k += kBlock)
+        s_rec[k / kSweepRecord][k % kSweepRecord] = __ldcg(a.sweep_tot + k);
+    __syncthreads();
+    const bool acc = a.accumulate == 1;
+    DevAccum &A = *a.acc;
+    const int t = threadIdx.x;
+    // lane t < HS_N_MOMENTS: moment t += x y over the sweeps, x and y from the record (y = 1 but for E^2)
+    constexpr int kE = kPartials, kMx = kPartials + 1;
+    if (t < HS_N_MOMENTS) {
+        if (acc) {
+            const int idx[HS_N_MOMENTS] = {kE, kE, kMx + 3, kMx + 4, kMx + 5, kMx, kMx + 1, kMx + 2, kMx + 6};
+            int at = 0;
+#pragma unroll
+            for (int q = 0; q < HS_N_MOMENTS; ++q) at = t == q ? idx[q] : at;
+            double m = A.moments[t];
+            for (int i = 0; i < n_slots; ++i) m = fma(s_rec[i][at], t == HS_SUM_E2 ? s_rec[i][at] : 1.0, m);
+            A.moments[t] = m;
+        }
+    } else if (t == HS_N_MOMENTS) {
+        if (acc) {
+            double n = A.count;
+            for (int i = 0; i < n_slots; ++i) n += 1.0;
+            A.count = n;
+        }
+    } else if (t == 32) {
+        double n = A.accepted;
+        for (int i = 0; i < n_slots; ++i) n += s_rec[i][4];
+        A.accepted = n;
+    } else if (t >= 64 && t < 64 + kPartials) {
+        A.sums[t - 64] = s_rec[n_slots - 1][t - 64];
+    } else if (t >= 96 && t < 96 + 8) {
+        if (acc) A.last[t - 96] = s_rec[n_slots - 1][kPartials + t - 96];
+    }
+}
+
+__global__ void __launch_bounds__(kBlock) fold_kernel(const PassArgs a) {
+    __shared__ int s_last;
+    pdl_enter();
     double tot[kPartials];
     slot_totals<kBlock>(a, blockIdx.x, tot);
     if (threadIdx.x == 0) {
@@ -772,26 +815,14 @@ __global__ void __launch_bounds__(kBlock) fold_sum_kernel(const PassArgs a) {
         for (int q = 0; q < kPartials; ++q) rec[q] = tot[q];
 #pragma unroll
         for (int q = 0; q < 8; ++q) rec[kPartials + q] = o[q];
+        __threadfence();
+        s_last = atomicAdd(&a.acc->done, 1u) == gridDim.x - 1u;
+        __threadfence();
     }
-}
-
-// ... and one thread applies the records to the accumulator in sweep order,
-// the accumulator held in registers over the group.
-__global__ void fold_apply_kernel(const PassArgs a, int n_slots) {
-    if (threadIdx.x != 0) return;
-    AccRegs R;
-    R.load(a.acc);
-    const bool acc = a.accumulate == 1;
-    for (int i = 0; i < n_slots; ++i) {
-        const double *rec = a.sweep_tot + (size_t)i * kSweepRecord;
-        double tot[kPartials], o[8];
-#pragma unroll
-        for (int q = 0; q < kPartials; ++q) tot[q] = rec[q];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) o[q] = rec[kPartials + q];
-        apply_sweep(R, tot, o, acc, acc);
-    }
-    R.store(a.acc);
+    __syncthreads();
+    if (!s_last) return;
+    fold_apply(a, (int)gridDim.x);
+    if (threadIdx.x == 0) a.acc->done = 0u;
 }
 
 // ----------------------------------------------------------------- init / layout
@@ -1108,11 +1139,7 @@ cudaError_t launch_pass_p(const Layout &L, const PassArgs &a, int n_blocks, cuda
 
 cudaError_t launch_fold(const PassArgs &a, int n_slots, cudaStream_t s) {
     if (n_slots < 1 || n_slots > kRingMax) return cudaErrorInvalidValue;
-    fold_sum_kernel<<<n_slots, kBlock, 0, s>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    fold_apply_kernel<<<1, 32, 0, s>>>(a, n_slots);
-    return cudaGetLastError();
+    return launch_pdl(fold_kernel, n_slots, kBlock, 0, s, a);
 }
 
 size_t storage_size(int precision) {
