@@ -537,11 +537,14 @@ int record_event(hs_lattice *h) {
     return HS_OK;
 }
 
-int check_device_error(hs_lattice *h) {
-    int err = 0;
-    HS_CUDA(cudaMemcpyAsync(&err, &h->acc->error, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+// The accumulator block of a lattice, once the work on its stream is done: one
+// copy of all of its fields, the latched error among them.  (Each copy to
+// host memory costs a round trip of its own, 10 us with its synchronisation;
+// reading the moments took two and a measurement three.)
+int read_accum(hs_lattice *h, DevAccum &out) {
+    HS_CUDA(cudaMemcpyAsync(&out, h->acc, sizeof(DevAccum), cudaMemcpyDeviceToHost, h->stream));
     HS_CUDA(cudaStreamSynchronize(h->stream));
-    if (err != 0) {
+    if (out.error != 0) {
         HS_CUDA(cudaMemsetAsync(&h->acc->error, 0, sizeof(int), h->stream));
         return fail(HS_E_TIMEOUT, "a bounded device-side wait timed out");
     }
@@ -1049,8 +1052,10 @@ int hs_get_sites(hs_lattice *h, int64_t n, const int64_t *sites, double *out) {
 
 int hs_read_sums(hs_lattice *h, double out[5]) {
     if (!h || !out) return fail(HS_E_INVALID, "null argument");
-    HS_CUDA(cudaMemcpyAsync(out, h->acc->sums, 5 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    return check_device_error(h);
+    DevAccum A;
+    const int st = read_accum(h, A);
+    if (st == HS_OK || st == HS_E_TIMEOUT) std::memcpy(out, A.sums, 5 * sizeof(double));
+    return st;
 }
 
 int hs_measure(hs_lattice *h, hs_measurement *out) {
@@ -1067,20 +1072,18 @@ int hs_measure(hs_lattice *h, hs_measurement *out) {
     a.accumulate = 0;
     a.n_blocks = hs::measure_blocks(h->L, h->n_sm, h->max_blocks);
     HS_CUDA(hs::launch_measure(h->precision, h->L, a, a.n_blocks, h->stream));
-    double last[8], accepted = 0.0;
-    HS_CUDA(cudaMemcpyAsync(last, h->acc->last, sizeof(last), cudaMemcpyDeviceToHost, h->stream));
-    HS_CUDA(cudaMemcpyAsync(&accepted, &h->acc->accepted, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    int st = check_device_error(h);
+    DevAccum A;
+    int st = read_accum(h, A);
     if (st) return st;
-    out->E = last[0];
-    out->M[0] = last[1];
-    out->M[1] = last[2];
-    out->M[2] = last[3];
-    out->absM = last[4];
-    out->M2 = last[5];
-    out->M4 = last[6];
+    out->E = A.last[0];
+    out->M[0] = A.last[1];
+    out->M[1] = A.last[2];
+    out->M[2] = A.last[3];
+    out->absM = A.last[4];
+    out->M2 = A.last[5];
+    out->M4 = A.last[6];
     const double attempts = (double)h->last_n_sweeps * (double)h->L.n_present;
-    out->accept_rate = attempts > 0 ? accepted / attempts : 0.0;
+    out->accept_rate = attempts > 0 ? A.accepted / attempts : 0.0;
     return HS_OK;
 }
 
@@ -1098,12 +1101,11 @@ int hs_reset_accumulator(hs_lattice *h) {
 
 int hs_read_accumulator(hs_lattice *h, double moments[HS_N_MOMENTS], int64_t *count) {
     if (!h || !moments || !count) return fail(HS_E_INVALID, "null argument");
-    double buf[HS_N_MOMENTS + 1];
-    HS_CUDA(cudaMemcpyAsync(buf, h->acc->moments, sizeof(buf), cudaMemcpyDeviceToHost, h->stream));
-    int st = check_device_error(h);
+    DevAccum A;
+    int st = read_accum(h, A);
     if (st) return st;
-    std::memcpy(moments, buf, sizeof(double) * HS_N_MOMENTS);
-    *count = (int64_t)buf[HS_N_MOMENTS];
+    std::memcpy(moments, A.moments, sizeof(double) * HS_N_MOMENTS);
+    *count = (int64_t)A.count;
     return HS_OK;
 }
 
