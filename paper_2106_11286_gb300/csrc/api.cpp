@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "batch.h"
+#include "cluster.h"
 #include "hs_impl.h"
 #include "slab.h"
 #include "upload.h"
@@ -205,6 +206,7 @@ struct hs_lattice {
     Layout L{};
     int n_blocks = 1;
     hs_launch req{};        // requested launch configuration (0 = automatic)
+    hs::ClusterPlan cluster{0, 0, 1};  // small lattices' automatic launch: a whole group of sweeps in one cluster
     int max_blocks = 1;     // capacity of the partials buffer
     int fold_ring = 1;      // sweeps per ring fold (slot sets of the partials buffer)
     double *partials = nullptr;
@@ -259,6 +261,9 @@ struct hs_lattice {
 
 namespace {
 
+// 1: the easy axis is (0, 0, 1) exactly
+int z_axis(const hs_lattice *h) { return h->p.e[0] == 0.0 && h->p.e[1] == 0.0 && h->p.e[2] == 1.0 ? 1 : 0; }
+
 PassArgs base_args(const hs_lattice *h) {
     PassArgs a{};
     const Layout &L = h->L;
@@ -296,7 +301,7 @@ PassArgs base_args(const hs_lattice *h) {
     a.replica = h->replica;
     a.sc_tab = h->sc_tab;
     a.tensor = h->tensor;
-    a.zaxis = (h->p.e[0] == 0.0 && h->p.e[1] == 0.0 && h->p.e[2] == 1.0) ? 1 : 0;
+    a.zaxis = z_axis(h);
     for (int q = 0; q < 6; ++q) {
         a.A[q] = h->tA[q];
         a.fA[q] = (float)h->tA[q];
@@ -430,6 +435,7 @@ int configure_launch(hs_lattice *h) {
         return fail(HS_E_INVALID, "a slab's sweep is in progress");
     const hs_launch &r = h->req;
     L.tensor = h->tensor;
+    h->cluster = hs::ClusterPlan{0, 0, 1};
     if (!L.structured) {
         L.kernel = hs::kTable;
         // request 1 = L2 prefetch of the next site's table row, 2 = off, 0 = automatic (on for FP32 tables of
@@ -505,6 +511,8 @@ int configure_launch(hs_lattice *h) {
     const int occ = std::min(hs::pass_occupancy(h->precision, L, 0), hs::pass_occupancy(h->precision, L, 1));
     if (bps <= 0 || bps > occ) bps = occ;
     h->n_blocks = std::min(hs::pass_blocks(h->precision, L, h->n_sm, bps), h->max_blocks);
+    if (r.kernel == HS_KERNEL_AUTO && r.vec_width == 0 && r.blocks_per_sm == 0 && r.prefetch == 0 && r.order == 0)
+        h->cluster = hs::cluster_plan(h->precision, L, z_axis(h));
     return clear_slab_sets(h);  // the parts' grids follow the launch configuration
 }
 
@@ -820,6 +828,18 @@ int hs_sweep(hs_lattice *h, double beta, int64_t n_sweeps) {
     a.accumulate = h->accumulate;
     // sweep s writes ring slot s mod ring; each full ring, and the rest after
     // the loop, is folded into the accumulator in sweep order
+    if (h->cluster.ctas > 0 && !h->timing) {  // (timing counts the colour passes' own launches)
+        a.n_blocks = h->cluster.ctas;
+        for (int64_t s = 0; s < n_sweeps;) {
+            const int k = (int)std::min<int64_t>(h->fold_ring, n_sweeps - s);
+            a.sweep = (uint32_t)(h->sweep + (uint64_t)s);
+            HS_CUDA(hs::launch_cluster(h->precision, h->L, h->cluster, a, k, h->stream));
+            HS_CUDA(hs::launch_fold(a, k, h->stream));
+            s += k;
+        }
+        h->sweep += (uint64_t)n_sweeps;
+        return HS_OK;
+    }
     int pending = 0;
     for (int64_t s = 0; s < n_sweeps; ++s) {
         for (int c = 0; c < h->L.n_colours; ++c)
@@ -1347,6 +1367,7 @@ std::vector<hs_launch> tune_candidates(hs_lattice *h) {
             for (int pf : {1, 2}) out.push_back({HS_KERNEL_TABLE, 1, b, 0, pf});
         return out;
     }
+    out.push_back(hs_launch{});  // the automatic launch (a small lattice's runs in one cluster)
     for (int v : {1, 2, 4, 8}) {
         if (!vec_ok(h, v)) continue;
         for (int b = 1; b <= 8; ++b)
