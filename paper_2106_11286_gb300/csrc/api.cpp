@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <array>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -206,7 +207,7 @@ struct hs_lattice {
     Layout L{};
     int n_blocks = 1;
     hs_launch req{};        // requested launch configuration (0 = automatic)
-    hs::ClusterPlan cluster{0, 0, 1};  // small lattices' automatic launch: a whole group of sweeps in one cluster
+    hs::GroupPlan group{0, 0, 1, false};  // small lattices' automatic launch: a whole group of sweeps at once
     int max_blocks = 1;     // capacity of the partials buffer
     int fold_ring = 1;      // sweeps per ring fold (slot sets of the partials buffer)
     double *partials = nullptr;
@@ -435,7 +436,7 @@ int configure_launch(hs_lattice *h) {
         return fail(HS_E_INVALID, "a slab's sweep is in progress");
     const hs_launch &r = h->req;
     L.tensor = h->tensor;
-    h->cluster = hs::ClusterPlan{0, 0, 1};
+    h->group = hs::GroupPlan{0, 0, 1, false};
     if (!L.structured) {
         L.kernel = hs::kTable;
         // request 1 = L2 prefetch of the next site's table row, 2 = off, 0 = automatic (on for FP32 tables of
@@ -512,7 +513,7 @@ int configure_launch(hs_lattice *h) {
     if (bps <= 0 || bps > occ) bps = occ;
     h->n_blocks = std::min(hs::pass_blocks(h->precision, L, h->n_sm, bps), h->max_blocks);
     if (r.kernel == HS_KERNEL_AUTO && r.vec_width == 0 && r.blocks_per_sm == 0 && r.prefetch == 0 && r.order == 0)
-        h->cluster = hs::cluster_plan(h->precision, L, z_axis(h));
+        h->group = hs::group_plan(h->precision, L, z_axis(h), h->n_blocks, h->n_sm);
     return clear_slab_sets(h);  // the parts' grids follow the launch configuration
 }
 
@@ -818,7 +819,8 @@ int hs_sweep(hs_lattice *h, double beta, int64_t n_sweeps) {
     if (h->L.slab && n_sweeps > 0)
         return fail(HS_E_INVALID, "a slab sweeps pass by pass (hs_sweep_pass), its halos refreshed in between");
     h->last_n_sweeps = n_sweeps;
-    HS_CUDA(cudaMemsetAsync(&h->acc->accepted, 0, sizeof(double), h->stream));
+    static_assert(offsetof(DevAccum, passed) == offsetof(DevAccum, accepted) + sizeof(double), "zeroed together");
+    HS_CUDA(cudaMemsetAsync(&h->acc->accepted, 0, sizeof(double) + sizeof(unsigned long long), h->stream));
     if (n_sweeps == 0 || h->L.n_present == 0) {
         h->sweep += (uint64_t)n_sweeps;
         return HS_OK;
@@ -828,13 +830,14 @@ int hs_sweep(hs_lattice *h, double beta, int64_t n_sweeps) {
     a.accumulate = h->accumulate;
     // sweep s writes ring slot s mod ring; each full ring, and the rest after
     // the loop, is folded into the accumulator in sweep order
-    if (h->cluster.ctas > 0 && !h->timing) {  // (timing counts the colour passes' own launches)
-        a.n_blocks = h->cluster.ctas;
+    if (h->group.ctas > 0 && !h->timing) {  // (timing counts the colour passes' own launches)
+        a.n_blocks = h->group.ctas;
         for (int64_t s = 0; s < n_sweeps;) {
             const int k = (int)std::min<int64_t>(h->fold_ring, n_sweeps - s);
             a.sweep = (uint32_t)(h->sweep + (uint64_t)s);
-            HS_CUDA(hs::launch_cluster(h->precision, h->L, h->cluster, a, k, h->stream));
+            HS_CUDA(hs::launch_group(h->precision, h->L, h->group, a, k, h->stream));
             HS_CUDA(hs::launch_fold(a, k, h->stream));
+            a.bar_base += (unsigned long long)h->group.ctas * (2 * k - 1);  // no barrier after a launch's last pass
             s += k;
         }
         h->sweep += (uint64_t)n_sweeps;
@@ -1367,7 +1370,7 @@ std::vector<hs_launch> tune_candidates(hs_lattice *h) {
             for (int pf : {1, 2}) out.push_back({HS_KERNEL_TABLE, 1, b, 0, pf});
         return out;
     }
-    out.push_back(hs_launch{});  // the automatic launch (a small lattice's runs in one cluster)
+    out.push_back(hs_launch{});  // the automatic launch (a small lattice's is one for a whole group of sweeps)
     for (int v : {1, 2, 4, 8}) {
         if (!vec_ok(h, v)) continue;
         for (int b = 1; b <= 8; ++b)

@@ -1,23 +1,32 @@
-// Sweeps of a small lattice inside one thread-block cluster (cluster.cu).
+// Sweeps of a small lattice, a group of them in one launch (cluster.cu).
 #pragma once
 
 #include "hs_impl.h"
 
 namespace hs {
 
-// The largest lattices that run in one cluster: beyond them the 16 SMs of a
-// cluster take longer over a pass than the whole device takes to launch it.
-constexpr int64_t kClusterSites = 65536;    // FP32, FP16
-constexpr int64_t kClusterSites64 = 16384;  // FP64
+// The largest lattices that run in one cluster: beyond them its 16 SMs take
+// longer over a pass than a barrier over the whole device costs (FP32 40^3: 7.5
+// us per sweep in the cluster, 5.5 on the grid; FP64 24^3: 10.4 against 8.9 for
+// 32^3 on the grid).
+constexpr int64_t kClusterSites = 32768;   // FP32, FP16
+constexpr int64_t kClusterSites64 = 8192;  // FP64
+// The largest that run as one cooperative launch: beyond them the launches
+// are a small part of a pass (times in cluster.cu).
+constexpr int64_t kGridSites = 3000000;    // FP32, FP16
+constexpr int64_t kGridSites64 = 1000000;  // FP64
 
-// CTAs (0: the launch chain instead) of how many threads, and sites per work item.
-struct ClusterPlan {
+// CTAs (0: the launch chain instead) of how many threads, sites per work item;
+// grid: a cooperative launch, else one cluster.
+struct GroupPlan {
     int ctas, threads, vec;
+    bool grid;
 };
-ClusterPlan cluster_plan(int precision, const Layout &L, int zaxis);
+GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, int n_sm);
 
-// n_sweeps sweeps from a.sweep on, sweep s to ring slot s; a.n_blocks = p.ctas.
-cudaError_t launch_cluster(int precision, const Layout &L, const ClusterPlan &p, const PassArgs &a, int n_sweeps,
-                           cudaStream_t s);
+// n_sweeps sweeps from a.sweep on, sweep s to ring slot s; a.n_blocks = p.ctas,
+// a.bar_base = arrivals already counted in a.acc->passed.
+cudaError_t launch_group(int precision, const Layout &L, const GroupPlan &p, const PassArgs &a, int n_sweeps,
+                         cudaStream_t s);
 
 }  // namespace hs

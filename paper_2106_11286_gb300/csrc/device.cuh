@@ -788,6 +788,47 @@ __device__ __forceinline__ void item_fields64(const Vec<double, V> (&o)[3], cons
     }
 }
 
+// The trials and acceptance uniforms of a work item's V sites, for a kernel
+// that draws them ahead of the item's loads (they need no spin).
+template <int P, int V>
+struct Trials {
+    float x[V], y[V], z[V], u[V];
+};
+template <int V>
+struct Trials<HS_FP64, V> {
+    Trial64 t[V];
+    uint32_t px[V], py[V];  // the acceptance uniform's words
+};
+
+template <int P, int V>
+__device__ __forceinline__ void draw_trials(const PassArgs &a, int c, uint32_t site0, uint32_t rank0, Trials<P, V> &d) {
+    if constexpr (P == HS_FP64) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            const uint32_t site = site0 + 2u * k;
+            d.t[k] = trial64(trial64_block(site, a.sweep, (uint32_t)c, 0u, a.replica, a.key0, a.key1), a.sc_tab);
+            const uint4 w = trial64_block(site, a.sweep, (uint32_t)c, 1u, a.replica, a.key0, a.key1);
+            d.px[k] = w.x;
+            d.py[k] = w.y;
+        }
+    } else if constexpr (V >= 2) {  // rank0 is even: rows hold a multiple of V sites
+#pragma unroll
+        for (int j = 0; j < V / 2; ++j) {
+            const uint4 w = trial_block((rank0 >> 1) + j, a.sweep, (uint32_t)c, a.replica, a.key0, a.key1);
+            float2 zi, vi, ui, x, y, z, u;
+            half_ints(w.x, w.y, zi.x, vi.x, ui.x);
+            half_ints(w.z, w.w, zi.y, vi.y, ui.y);
+            trial32<P, float2>(zi, vi, ui, x, y, z, u);
+            d.x[2 * j] = x.x, d.x[2 * j + 1] = x.y;
+            d.y[2 * j] = y.x, d.y[2 * j + 1] = y.y;
+            d.z[2 * j] = z.x, d.z[2 * j + 1] = z.y;
+            d.u[2 * j] = u.x, d.u[2 * j + 1] = u.y;
+        }
+    } else {
+        draw_trial_rank<P>(rank0, a.sweep, (uint32_t)c, a.replica, a.key0, a.key1, d.x[0], d.y[0], d.z[0], d.u[0]);
+    }
+}
+
 // Where a work item's operands lie, for the few sites whose FP32 decision is
 // open: the other colour's planes and the item's first element.
 struct ItemSource {
@@ -830,17 +871,25 @@ __device__ __noinline__ bool accept_wide(double sx, double sy, double sz, double
 // update_item_h); ZAX as in metropolis.  Spins, trials and sums are FP64; the
 // decision is the FP64 rule's, taken from FP32 values wherever their error
 // bound settles it (decide64).
-template <int V, bool MEAS, bool TEN, bool ZAX, bool CG>
+template <int V, bool MEAS, bool TEN, bool ZAX, bool CG, bool PRE>
 __device__ __forceinline__ bool update_fp64(Vec<double, V> (&s)[3], const Field64<V> &F, uint32_t site0, int c,
                                             const PassArgs &a, double J, double K, double ex, double ey, double ez,
-                                            double beta, SiteAcc<HS_FP64> &acc, const ItemSource &src) {
+                                            double beta, SiteAcc<HS_FP64> &acc, const ItemSource &src,
+                                            const Trials<HS_FP64, V> *pre) {
     bool any = false;
 #pragma unroll
     for (int k = 0; k < V; ++k) {
-        const uint32_t site = site0 + 2u * k;
-        const Trial64 t =
-            trial64(trial64_block(site, a.sweep, (uint32_t)c, 0u, a.replica, a.key0, a.key1), a.sc_tab);
-        const uint4 pw = trial64_block(site, a.sweep, (uint32_t)c, 1u, a.replica, a.key0, a.key1);
+        Trial64 t;
+        uint2 pw;
+        if constexpr (PRE) {
+            t = pre->t[k];
+            pw = make_uint2(pre->px[k], pre->py[k]);
+        } else {
+            const uint32_t site = site0 + 2u * k;
+            t = trial64(trial64_block(site, a.sweep, (uint32_t)c, 0u, a.replica, a.key0, a.key1), a.sc_tab);
+            const uint4 w = trial64_block(site, a.sweep, (uint32_t)c, 1u, a.replica, a.key0, a.key1);
+            pw = make_uint2(w.x, w.y);
+        }
         const float uf = (float)(pw.x >> 8) * 0x1p-24f;  // P's top 24 bits
         double sx = s[0].v[k], sy = s[1].v[k], sz = s[2].v[k];
         bool ac;
@@ -901,10 +950,10 @@ __device__ __forceinline__ bool update_fp64(Vec<double, V> (&s)[3], const Field6
 // (see update_item_h); ZAX as in site_math32.
 // KZ (with ZAX): K = +0, whose energy share -K (S.e)^2 is -0 (written as such,
 // so every sum takes the same values; adding -0 changes none).
-template <int P, int V, bool MEAS, bool TEN, bool ZAX, bool KZ = false>
+template <int P, int V, bool MEAS, bool TEN, bool ZAX, bool KZ = false, bool PRE = false>
 __device__ __forceinline__ bool update_f32(Vec<typename Tr<P>::S, V> (&s)[3], const float (&h)[3][V], uint32_t rank0,
                                            int c, const PassArgs &a, float J, float K, float ex, float ey, float ez,
-                                           float beta, SiteAcc<P> &acc) {
+                                           float beta, SiteAcc<P> &acc, const Trials<P, V> *pre = nullptr) {
     using S = typename Tr<P>::S;
     using C = float;
     bool any = false;
@@ -934,16 +983,23 @@ __device__ __forceinline__ bool update_f32(Vec<typename Tr<P>::S, V> (&s)[3], co
         }
     };
     // ranks of the item's sites in their colour class: rank0 + k
-    if (V >= 2 && (rank0 & 1u) == 0u) {
+    if (V >= 2 && (PRE || (rank0 & 1u) == 0u)) {
 #pragma unroll
         for (int j = 0; j < V / 2; ++j) {  // one Philox block and packed arithmetic per pair
             const int k0 = 2 * j, k1 = 2 * j + 1;
-            const uint4 w = trial_block((rank0 >> 1) + j, a.sweep, (uint32_t)c, a.replica, a.key0, a.key1);
-            float2 zi, vi, ui;
-            half_ints(w.x, w.y, zi.x, vi.x, ui.x);
-            half_ints(w.z, w.w, zi.y, vi.y, ui.y);
             float2 tx, ty, tz, u;
-            trial32<P, float2>(zi, vi, ui, tx, ty, tz, u);
+            if constexpr (PRE) {
+                tx = make_float2(pre->x[k0], pre->x[k1]);
+                ty = make_float2(pre->y[k0], pre->y[k1]);
+                tz = make_float2(pre->z[k0], pre->z[k1]);
+                u = make_float2(pre->u[k0], pre->u[k1]);
+            } else {
+                const uint4 w = trial_block((rank0 >> 1) + j, a.sweep, (uint32_t)c, a.replica, a.key0, a.key1);
+                float2 zi, vi, ui;
+                half_ints(w.x, w.y, zi.x, vi.x, ui.x);
+                half_ints(w.z, w.w, zi.y, vi.y, ui.y);
+                trial32<P, float2>(zi, vi, ui, tx, ty, tz, u);
+            }
             float2 hp[3];
 #pragma unroll
             for (int q = 0; q < 3; ++q) hp[q] = make_float2(h[q][k0], h[q][k1]);
@@ -983,7 +1039,11 @@ __device__ __forceinline__ bool update_f32(Vec<typename Tr<P>::S, V> (&s)[3], co
 #pragma unroll
         for (int k = 0; k < V; ++k) {
             float tx, ty, tz, u;
-            draw_trial_rank<P>(rank0 + k, a.sweep, (uint32_t)c, a.replica, a.key0, a.key1, tx, ty, tz, u);
+            if constexpr (PRE) {
+                tx = pre->x[k], ty = pre->y[k], tz = pre->z[k], u = pre->u[k];
+            } else {
+                draw_trial_rank<P>(rank0 + k, a.sweep, (uint32_t)c, a.replica, a.key0, a.key1, tx, ty, tz, u);
+            }
             single(k, tx, ty, tz, u);
         }
     }
@@ -1018,33 +1078,38 @@ __device__ __forceinline__ void fields_of(const Vec<typename Tr<P>::S, V> (&o)[3
 // with no branch (the FP32 register stencil's form); AX = 2: the same with
 // K = +0 (the FP32 and FP16 batch kernels); AX = 0: FP64 and FP16 decide per
 // work item from PassArgs::zaxis, FP32 takes the general products.
-// oth, b0: where the item's neighbours lie (FP64; CG as in ld_val).
-template <int P, int V, bool MEAS, bool TEN = false, int AX = 0, bool CG = false>
+// oth, b0: where the item's neighbours lie (FP64; CG as in ld_val).  PRE: the
+// trials are drawn already (pre).
+template <int P, int V, bool MEAS, bool TEN = false, int AX = 0, bool CG = false, bool PRE = false>
 __device__ __forceinline__ bool update_item_h(Vec<typename Tr<P>::S, V> (&s)[3],
                                               const typename ItemField<P, V>::T &h, uint32_t site0, uint32_t rank0,
                                               int c, const PassArgs &a, typename Tr<P>::C J, typename Tr<P>::C K,
                                               typename Tr<P>::C ex, typename Tr<P>::C ey, typename Tr<P>::C ez,
                                               typename Tr<P>::C beta, SiteAcc<P> &acc,
-                                              const typename Tr<P>::S *const (&oth)[3], uint32_t b0) {
+                                              const typename Tr<P>::S *const (&oth)[3], uint32_t b0,
+                                              const Trials<P, V> *pre = nullptr) {
     if constexpr (P == HS_FP64) {
         // one uniform branch per work item: the item body with S.e = S_z
         // (e = (0, 0, 1)) or with the general dot products
         const ItemSource src{{oth[0], oth[1], oth[2]}, b0};
         if constexpr (!TEN)
             if (a.zaxis)
-                return update_fp64<V, MEAS, false, true, CG>(s, h, site0, c, a, J, K, ex, ey, ez, beta, acc, src);
-        return update_fp64<V, MEAS, TEN, false, CG>(s, h, site0, c, a, J, K, ex, ey, ez, beta, acc, src);
+                return update_fp64<V, MEAS, false, true, CG, PRE>(s, h, site0, c, a, J, K, ex, ey, ez, beta, acc, src,
+                                                                  pre);
+        return update_fp64<V, MEAS, TEN, false, CG, PRE>(s, h, site0, c, a, J, K, ex, ey, ez, beta, acc, src, pre);
     } else {
         if constexpr (AX >= 1 && !TEN)
-            return update_f32<P, V, MEAS, false, true, AX == 2>(s, h, rank0, c, a, J, K, ex, ey, ez, beta, acc);
+            return update_f32<P, V, MEAS, false, true, AX == 2, PRE>(s, h, rank0, c, a, J, K, ex, ey, ez, beta, acc,
+                                                                     pre);
         // FP16 (bound by instruction issue, its loads decoupled by the
         // pipelined landing slots) takes the same branch; the FP32 register
         // stencil, bound by load latency, measured slower with it (the branch
         // between an item's loads and its arithmetic costs more than the three
         // instructions per site it saves) and keeps the general products
         if constexpr (!TEN && P == HS_FP16)
-            if (a.zaxis) return update_f32<P, V, MEAS, false, true>(s, h, rank0, c, a, J, K, ex, ey, ez, beta, acc);
-        return update_f32<P, V, MEAS, TEN, false>(s, h, rank0, c, a, J, K, ex, ey, ez, beta, acc);
+            if (a.zaxis)
+                return update_f32<P, V, MEAS, false, true, false, PRE>(s, h, rank0, c, a, J, K, ex, ey, ez, beta, acc, pre);
+        return update_f32<P, V, MEAS, TEN, false, false, PRE>(s, h, rank0, c, a, J, K, ex, ey, ez, beta, acc, pre);
     }
 }
 
@@ -1128,14 +1193,12 @@ __device__ __forceinline__ ItemOffsets item_offsets(const PassArgs &a, uint32_t 
     return o;
 }
 
-// Load the operands of the work item at row (y, z), vector xv.
+// Load a work item's operands from their offsets.
 template <int P, int V, bool CG = false>
-__device__ __forceinline__ void load_item_at(const PassArgs &a, uint32_t y, uint32_t z, uint32_t xv,
-                                             const typename Tr<P>::S *const (&own)[3],
-                                             const typename Tr<P>::S *const (&oth)[3], StencilItem<P, V> &it) {
+__device__ __forceinline__ void load_item_from(const ItemOffsets &f, const typename Tr<P>::S *const (&own)[3],
+                                               const typename Tr<P>::S *const (&oth)[3], StencilItem<P, V> &it) {
     using S = typename Tr<P>::S;
     using VT = Vec<S, V>;
-    const ItemOffsets f = item_offsets<V>(a, y, z, xv);
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
         it.s[q] = ld_val<VT, CG>(reinterpret_cast<const VT *>(own[q] + f.b0));
@@ -1150,6 +1213,14 @@ __device__ __forceinline__ void load_item_at(const PassArgs &a, uint32_t y, uint
     it.p = f.p;
     it.site0 = f.site0;
     it.rank0 = f.rank0;
+}
+
+// Load the operands of the work item at row (y, z), vector xv.
+template <int P, int V, bool CG = false>
+__device__ __forceinline__ void load_item_at(const PassArgs &a, uint32_t y, uint32_t z, uint32_t xv,
+                                             const typename Tr<P>::S *const (&own)[3],
+                                             const typename Tr<P>::S *const (&oth)[3], StencilItem<P, V> &it) {
+    load_item_from<P, V, CG>(item_offsets<V>(a, y, z, xv), own, oth, it);
 }
 
 // The work item with linear index t = (z Ly + y) (Lh/V) + xv (rev - t in a

@@ -57,6 +57,7 @@ struct DevAccum {
     double moments[HS_N_MOMENTS];
     double count;          // accumulated sweeps
     double accepted;       // accepted moves since the last hs_sweep began
+    unsigned long long passed;  // CTA arrivals at the pass barrier of a cooperative sweep launch since then
     double last[8];        // E, Mx, My, Mz, |M|, M2, M4, |M.e| of the last finalised reduction
     unsigned int done;     // CTA arrival counter of the finishing pass
     int error;             // latched device error code (0 = none)
@@ -111,6 +112,7 @@ struct PassArgs {
                             // 2: measure only (the sums; a slab whose moments come from all slabs' sums)
     double n_present;
     DevAccum *acc;
+    unsigned long long bar_base;  // cooperative sweep launch: arrivals counted before it
 };
 
 // codes as in hs_kernel (include/hs.h)

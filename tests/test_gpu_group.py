@@ -1,0 +1,46 @@
+"""The automatic launch of small lattices (a whole group of sweeps in one
+cluster, or in one cooperative launch) against the launch chain: the same
+spins bit for bit, the same accepted moves, and moments that differ by FP64
+rounding at most -- FP32 / FP16 sums are grouped alike, FP64 ones are added in
+another order, 10^4 terms of equal sign: below 1e-12.
+
+Sizes at the edges of the choice (32768 and 8192 sites, 3.0 and 1.0 million),
+of the warps and CTAs, of one or several items per thread, and of the vector
+widths; 70 sweeps, more than one group of 64, then one more call.
+"""
+import numpy as np
+import pytest
+
+from paper_2106_11286_gb300 import hs
+
+pytestmark = pytest.mark.gpu
+
+A6 = (0.1, -0.2, 0.05, 0.03, -0.04, 0.02)
+DIMS = [(2, 2, 2), (10, 6, 4), (12, 10, 14), (16, 16, 16), (32, 16, 16), (34, 16, 16), (64, 32, 16), (66, 32, 16),
+        (72, 64, 66)]
+LARGE = [(250, 62, 64), (128, 128, 182), (256, 184, 64)]
+
+
+def _run(dims, precision, e, K, tensor, meas, chain, sweeps):
+    with hs.Lattice("sc", dims=dims, precision=precision, seed=5, K=K, e=e, A=A6 if tensor else None) as lat:
+        if chain:
+            lat.set_launch(kernel="stencil")
+        lat.init()
+        lat.accumulate(meas)
+        for n in sweeps:
+            lat.sweep(0.8, n)
+        moments, count = lat.read_accumulator()
+        return lat.get_spins(), moments, count, lat.measure()["accept_rate"], lat.info.sweep
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("dims", DIMS + LARGE)
+@pytest.mark.parametrize("e,K,tensor,meas", [((0, 0, 1), 0.0, False, True), ((0.3, -0.2, 1.0), 0.3, False, True),
+                                             ((0, 0, 1), 0.1, True, True), ((0, 0, 1), 0.1, False, False)])
+def test_group_equals_the_launch_chain(precision, dims, e, K, tensor, meas):
+    sweeps = (3, 1) if dims in LARGE else (70, 1)
+    got = _run(dims, precision, e, K, tensor, meas, False, sweeps)
+    want = _run(dims, precision, e, K, tensor, meas, True, sweeps)
+    np.testing.assert_array_equal(got[0], want[0])
+    assert got[2:] == want[2:]
+    np.testing.assert_allclose(got[1], want[1], rtol=0, atol=1e-12 * max(1.0, np.abs(want[1]).max()))
