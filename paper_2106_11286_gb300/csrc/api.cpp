@@ -832,12 +832,13 @@ int hs_sweep(hs_lattice *h, double beta, int64_t n_sweeps) {
     // the loop, is folded into the accumulator in sweep order
     if (h->group.ctas > 0 && !h->timing) {  // (timing counts the colour passes' own launches)
         a.n_blocks = h->group.ctas;
+        unsigned long long arrivals = 0;
         for (int64_t s = 0; s < n_sweeps;) {
             const int k = (int)std::min<int64_t>(h->fold_ring, n_sweeps - s);
             a.sweep = (uint32_t)(h->sweep + (uint64_t)s);
-            HS_CUDA(hs::launch_group(h->precision, h->L, h->group, a, k, h->stream));
+            HS_CUDA(hs::launch_group(h->precision, h->L, h->group, a, k, arrivals, h->stream));
             HS_CUDA(hs::launch_fold(a, k, h->stream));
-            a.bar_base += (unsigned long long)h->group.ctas * (2 * k - 1);  // no barrier after a launch's last pass
+            arrivals += (unsigned long long)h->group.ctas * (2 * k - 1);  // no barrier after a launch's last pass
             s += k;
         }
         h->sweep += (uint64_t)n_sweeps;

@@ -145,7 +145,8 @@ struct PassBarrier {
 // Work item t of a pass belongs to thread t mod (threads of the grid, which in
 // a cluster launch is the cluster).
 template <int P, int V, bool MEAS, int AX, bool TEN, bool GRID>
-__device__ __forceinline__ void sweep_group(const PassArgs &args, void *planes, int n_sweeps, int alternate, int depth) {
+__device__ __forceinline__ void sweep_group(const PassArgs &args, void *planes, int n_sweeps, int alternate, int depth,
+                                            unsigned long long arrivals) {
     using S = typename Tr<P>::S;
     using C = typename Tr<P>::C;
     using VT = Vec<S, V>;
@@ -157,7 +158,7 @@ __device__ __forceinline__ void sweep_group(const PassArgs &args, void *planes, 
     held.depth = depth;
     held.v = reinterpret_cast<double *>(cluster_smem);
     held.n = reinterpret_cast<unsigned *>(held.v + (size_t)depth * 4 * held.units);
-    PassBarrier<GRID> bar{&a.acc->passed, a.bar_base, &a.acc->error};
+    PassBarrier<GRID> bar{&a.acc->passed, arrivals, &a.acc->error};
     const uint32_t nxv = a.Lh / V;
     const uint32_t n_items = (uint32_t)a.Lz * a.Ly * nxv;
     const size_t plane = (size_t)a.Lz * a.Ly * a.Lh;
@@ -273,13 +274,13 @@ template <int P, int V, bool MEAS, int AX, bool TEN>
 __global__ void __launch_bounds__(kClusterThreads, 1) sc_cluster_kernel(const PassArgs args, void *planes, int n_sweeps,
                                                                         int alternate, int depth) {
     pdl_enter();
-    sweep_group<P, V, MEAS, AX, TEN, false>(args, planes, n_sweeps, alternate, depth);
+    sweep_group<P, V, MEAS, AX, TEN, false>(args, planes, n_sweeps, alternate, depth, 0ull);
 }
 
 template <int P, int V, bool MEAS, int AX, bool TEN>
 __global__ void __launch_bounds__(kBlock, 2) sc_grid_kernel(const PassArgs args, void *planes, int n_sweeps,
-                                                            int alternate, int depth) {
-    sweep_group<P, V, MEAS, AX, TEN, true>(args, planes, n_sweeps, alternate, depth);
+                                                            int alternate, int depth, unsigned long long arrivals) {
+    sweep_group<P, V, MEAS, AX, TEN, true>(args, planes, n_sweeps, alternate, depth, arrivals);
 }
 
 // The variants of one precision and width: the tensor term, or FP32's S.e = S_z.
@@ -401,7 +402,7 @@ GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, in
 }
 
 cudaError_t launch_group(int precision, const Layout &L, const GroupPlan &p, const PassArgs &a, int n_sweeps,
-                         cudaStream_t s) {
+                         unsigned long long arrivals, cudaStream_t s) {
     const void *k = group_kernel(precision, p, a.accumulate != 0, L.tensor != 0, a.zaxis != 0);
     if (!k || n_sweeps < 1) return cudaErrorInvalidValue;
     PassArgs args = a;
@@ -412,7 +413,7 @@ cudaError_t launch_group(int precision, const Layout &L, const GroupPlan &p, con
     cudaLaunchAttribute attr[2];
     group_config(cfg, attr, precision, p, s);
     int depth = held_passes(precision, p.threads);
-    void *params[] = {&args, &planes, &n_sweeps, &alternate, &depth};
+    void *params[] = {&args, &planes, &n_sweeps, &alternate, &depth, &arrivals};  // a cluster's kernel takes the first five
     return cudaLaunchKernelExC(&cfg, k, params);
 }
 

@@ -25,8 +25,8 @@ struct GroupPlan {
 GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, int n_sm);
 
 // n_sweeps sweeps from a.sweep on, sweep s to ring slot s; a.n_blocks = p.ctas,
-// a.bar_base = arrivals already counted in a.acc->passed.
+// arrivals: those already counted in a.acc->passed.
 cudaError_t launch_group(int precision, const Layout &L, const GroupPlan &p, const PassArgs &a, int n_sweeps,
-                         cudaStream_t s);
+                         unsigned long long arrivals, cudaStream_t s);
 
 }  // namespace hs

@@ -482,32 +482,30 @@ __device__ __forceinline__ double warp_sum(double v) {
 // measurement), executed by one whole CTA: every CTA's partials of every
 // partial set not in a.skip_sets, summed in a fixed order (so the FP64
 // totals do not depend on scheduling); the result is valid in thread 0.
+// One warp per quantity: the FP64 pipe takes 16 cycles for a warp's addition,
+// so the shuffle trees (5 additions each) are taken once per quantity and not
+// once per warp and quantity (120 against 320 such additions for 608 CTAs'
+// partials and 8 warps).
 template <int NT = kBlock>
 __device__ void slot_totals(const PassArgs &a, int slot, double (&tot)[kPartials]) {
-    __shared__ double s_fin[NT / 32][kPartials];
-    double t[kPartials] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    const double *base = a.partials + (size_t)slot * a.n_colours * a.n_blocks * kPartials;
-    for (int p = 0; p < a.n_colours; ++p) {
-        if ((a.skip_sets >> p) & 1ull) continue;
-        for (int b = threadIdx.x; b < a.n_blocks; b += NT) {
-            const double *ps = base + ((size_t)p * a.n_blocks + b) * kPartials;
-#pragma unroll
-            for (int q = 0; q < kPartials; ++q) t[q] += __ldcg(ps + q);
-        }
-    }
+    __shared__ double s_fin[kPartials];
+    constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < kPartials; ++q) t[q] = warp_sum(t[q]);
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < kPartials; ++q) s_fin[warp][q] = t[q];
+    const double *base = a.partials + (size_t)slot * a.n_colours * a.n_blocks * kPartials;
+    for (int q = warp; q < kPartials; q += NW) {
+        double t = 0.0;
+        for (int p = 0; p < a.n_colours; ++p) {
+            if ((a.skip_sets >> p) & 1ull) continue;
+            const double *ps = base + (size_t)p * a.n_blocks * kPartials + q;
+#pragma unroll 4
+            for (int b = lane; b < a.n_blocks; b += 32) t += __ldcg(ps + (size_t)b * kPartials);
+        }
+        t = warp_sum(t);
+        if (lane == 0) s_fin[q] = t;
+    }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < kPartials; ++q) tot[q] = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < NT / 32; ++w)
-#pragma unroll
-            for (int q = 0; q < kPartials; ++q) tot[q] += s_fin[w][q];
+    for (int q = 0; q < kPartials; ++q) tot[q] = s_fin[q];
 }
 
 // Eq. 2 with |S| = 1 from one sweep's totals: o = E, Mx, My, Mz, |M|, M2, M4,
@@ -1078,7 +1076,7 @@ __device__ __forceinline__ void fields_of(const Vec<typename Tr<P>::S, V> (&o)[3
 // with no branch (the FP32 register stencil's form); AX = 2: the same with
 // K = +0 (the FP32 and FP16 batch kernels); AX = 0: FP64 and FP16 decide per
 // work item from PassArgs::zaxis, FP32 takes the general products.
-// oth, b0: where the item's neighbours lie (FP64; CG as in ld_val).  PRE: the
+// oth, b0: where the item's neighbours lie (FP64 only, which may read them again; CG as in ld_val).  PRE: the
 // trials are drawn already (pre).
 template <int P, int V, bool MEAS, bool TEN = false, int AX = 0, bool CG = false, bool PRE = false>
 __device__ __forceinline__ bool update_item_h(Vec<typename Tr<P>::S, V> (&s)[3],
@@ -1086,7 +1084,7 @@ __device__ __forceinline__ bool update_item_h(Vec<typename Tr<P>::S, V> (&s)[3],
                                               int c, const PassArgs &a, typename Tr<P>::C J, typename Tr<P>::C K,
                                               typename Tr<P>::C ex, typename Tr<P>::C ey, typename Tr<P>::C ez,
                                               typename Tr<P>::C beta, SiteAcc<P> &acc,
-                                              const typename Tr<P>::S *const (&oth)[3], uint32_t b0,
+                                              const typename Tr<P>::S *const *oth = nullptr, uint32_t b0 = 0,
                                               const Trials<P, V> *pre = nullptr) {
     if constexpr (P == HS_FP64) {
         // one uniform branch per work item: the item body with S.e = S_z
@@ -1123,7 +1121,8 @@ __device__ __forceinline__ bool update_item(Vec<typename Tr<P>::S, V> (&s)[3], c
                                             uint32_t p, uint32_t site0, uint32_t rank0, int c, const PassArgs &a,
                                             typename Tr<P>::C J, typename Tr<P>::C K, typename Tr<P>::C ex,
                                             typename Tr<P>::C ey, typename Tr<P>::C ez, typename Tr<P>::C beta,
-                                            SiteAcc<P> &acc, const typename Tr<P>::S *const (&oth)[3], uint32_t b0) {
+                                            SiteAcc<P> &acc, const typename Tr<P>::S *const *oth = nullptr,
+                                            uint32_t b0 = 0) {
     typename ItemField<P, V>::T h;
     fields_of<P, V, MEAS, TEN>(o, nym, nyp, nzm, nzp, ed, p, c, h);
     return update_item_h<P, V, MEAS, TEN, AX, CG>(s, h, site0, rank0, c, a, J, K, ex, ey, ez, beta, acc, oth, b0);

@@ -96,9 +96,10 @@ struct PassArgs {
     double A[6];            // its symmetric tensor (xx, yy, zz, xy, xz, yz)
     float fA[6];
     const ulonglong2 *sc_tab;  // FP64 trial: sin, cos(pi j / 4096) in units of 2^-63, j = 0..2047
-    float fdelta;           // FP64: bound on the error of the FP32 form of beta dH (decision_band)
     int zaxis;              // 1: e = (0, 0, 1) exactly (the FP64 stencil takes S.e = S_z)
     uint32_t key0, key1, replica, sweep;
+    float fdelta;           // FP64: bound on the error of the FP32 form of beta dH (decision_band); in what was
+                            // padding: the FP32 stencil measured 4 % slower with the words before it shifted
     double *partials;       // [ring slots][n_colours][n_blocks][kPartials]; a slab has kSlabSets sets per colour
                             // (pass = kSlabSets colour + set, n_colours = 2 kSlabSets); a launch of fewer CTAs
                             // than n_blocks leaves the rest of its set zero
@@ -112,7 +113,6 @@ struct PassArgs {
                             // 2: measure only (the sums; a slab whose moments come from all slabs' sums)
     double n_present;
     DevAccum *acc;
-    unsigned long long bar_base;  // cooperative sweep launch: arrivals counted before it
 };
 
 // codes as in hs_kernel (include/hs.h)

@@ -71,8 +71,14 @@ __global__ void __launch_bounds__(kBlock, 2) sc_pass_kernel(const PassArgs a) {
     SiteAcc<P> acc;
     const uint32_t stride = gridDim.x * blockDim.x;
     auto compute = [&](StencilItem<P, V> &it) {
-        if (update_item<P, V, MEAS, TEN, AX>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0, it.rank0,
-                                             c, a, J, K, ex, ey, ez, beta, acc, oth, it.b0)) {
+        bool any;
+        if constexpr (P == HS_FP64)
+            any = update_item<P, V, MEAS, TEN, AX>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0,
+                                                   it.rank0, c, a, J, K, ex, ey, ez, beta, acc, oth, it.b0);
+        else
+            any = update_item<P, V, MEAS, TEN, AX>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0,
+                                                   it.rank0, c, a, J, K, ex, ey, ez, beta, acc);
+        if (any) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) *reinterpret_cast<VT *>(own_w[q] + it.b0) = it.s[q];
         }
@@ -782,6 +788,7 @@ __device__ void fold_apply(const PassArgs &a, int n_slots) {
 #pragma unroll
             for (int q = 0; q < HS_N_MOMENTS; ++q) at = t == q ? idx[q] : at;
             double m = A.moments[t];
+#pragma unroll 8
             for (int i = 0; i < n_slots; ++i) m = fma(s_rec[i][at], t == HS_SUM_E2 ? s_rec[i][at] : 1.0, m);
             A.moments[t] = m;
         }
@@ -793,6 +800,7 @@ __device__ void fold_apply(const PassArgs &a, int n_slots) {
         }
     } else if (t == 32) {
         double n = A.accepted;
+#pragma unroll 8
         for (int i = 0; i < n_slots; ++i) n += s_rec[i][4];
         A.accepted = n;
     } else if (t >= 64 && t < 64 + kPartials) {
