@@ -92,6 +92,7 @@ __device__ void reduce_held(const PassArgs &a, const PassSums &h, int used, int 
             out[i * next + q] = t;
         }
     }
+    __syncthreads();  // the slots are written again by warps that need not wait for this one at the pass's barrier
 }
 
 constexpr long long kBarrierCycles = 2000000000LL;  // about one second
@@ -205,7 +206,6 @@ __device__ __forceinline__ void sweep_group(const PassArgs &args, void *planes, 
         if (lane == 0) held.n[used * held.warps + warp] = n;
         sum[0] = sum[1] = sum[2] = sum[3] = 0.0;
         n = 0;
-        // (the slots are written again after the barrier, by when every warp has read them)
         if (++used == depth || pass == 2 * n_sweeps - 1) {
             reduce_held<P>(a, held, used, pass);
             used = 0;
