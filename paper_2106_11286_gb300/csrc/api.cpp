@@ -1502,6 +1502,9 @@ struct hs_batch {
                                                    // 2: resident (one CTA per member, in shared memory)
     size_t resident_bytes = 0;                     // the largest member's six planes
     int precision = HS_FP32;                       // every member's
+    hs::BatchClusters clusters{0, 0};              // schedule 2 by clusters (FP64 batches of few small members)
+    double *d_group = nullptr;                     // their sums
+    hs::FastDiv *d_rows = nullptr;                 // their members' row divisions
     ~hs_batch() {
         cudaStreamSynchronize(stream);
         if (exec) cudaGraphExecDestroy(exec);
@@ -1512,7 +1515,11 @@ struct hs_batch {
         cudaFree(d_slots);
         cudaFree(d_bar);
         cudaFree(d_error);
+        cudaFree(d_group);
+        cudaFree(d_rows);
     }
+    // schedule 2 can run: every member in one CTA's shared memory, or in a cluster of its own
+    bool resident_ok() const { return clusters.ctas > 0 || resident_bytes <= hs::batch_resident_limit(precision); }
 };
 
 namespace {
@@ -1530,6 +1537,8 @@ hs::BatchArgs batch_args(const hs_batch *b, int n_total, int n_equil) {
     a.n_equil = n_equil;
     a.zaxis_all = 1;
     a.kzero_all = 1;
+    a.group = b->d_group;
+    a.member_rows = b->d_rows;
     for (const hs::BatchMember &m : b->host_members) {
         a.zaxis_all &= m.zaxis;
         a.kzero_all &= (m.K == 0.0 && !std::signbit(m.K)) ? 1 : 0;
@@ -1774,6 +1783,22 @@ int hs_batch_create(hs_batch **out, hs_lattice *const *members, int n_members) {
     // many small members: the resident schedule (measured 3.2x the persistent one on 304 members of 16^3,
     // 2.5x on 152 of 24^3, 1.2x on 16 of 24^3, which leave most SMs idle)
     if (n_members >= kResidentMinMembers && b->resident_bytes <= hs::batch_resident_limit(precision)) b->schedule = 2;
+    // FP64 batches of few small members: a cluster each
+    int64_t max_sites = 0;
+    for (const hs_lattice *h : b->members) max_sites = std::max(max_sites, h->L.n_sites);
+    b->clusters = hs::batch_cluster_plan(precision, n_members, max_sites, members[0]->n_sm);
+    if (b->clusters.ctas > 0) {
+        std::vector<hs::FastDiv> rows;
+        for (const hs_lattice *h : b->members) rows.emplace_back((uint32_t)h->L.Lh);
+        if ((e = cudaMalloc(&b->d_group, hs::batch_cluster_bytes(n_members, b->clusters))) != cudaSuccess ||
+            (e = cudaMalloc(&b->d_rows, rows.size() * sizeof(hs::FastDiv))) != cudaSuccess ||
+            (e = cudaMemcpy(b->d_rows, rows.data(), rows.size() * sizeof(hs::FastDiv), cudaMemcpyHostToDevice)) !=
+                cudaSuccess) {
+            delete b;
+            return cuda_fail(e, "cudaMalloc(batch)");
+        }
+        b->schedule = 2;
+    }
     *out = b;
     return HS_OK;
 }
@@ -1813,8 +1838,11 @@ int hs_batch_run(hs_batch *b, const double *betas, int64_t n_sweeps, int64_t n_e
         for (int r = 0; r < n; ++r) b->members[r]->sweep += (uint64_t)n_total;
         return HS_OK;
     }
-    if (b->schedule == 2) {  // one launch: every member resident in its CTA's shared memory
-        HS_CUDA(hs::launch_batch_resident(b->precision, args, b->resident_bytes, b->stream));
+    if (b->schedule == 2) {  // every member in a cluster of its own, or resident in its CTA's shared memory
+        if (b->clusters.ctas > 0)
+            HS_CUDA(hs::launch_batch_clusters(args, b->clusters, b->stream));
+        else
+            HS_CUDA(hs::launch_batch_resident(b->precision, args, b->resident_bytes, b->stream));
         for (int r = 0; r < n; ++r) b->members[r]->sweep += (uint64_t)n_total;
         return HS_OK;
     }
@@ -1906,7 +1934,7 @@ int hs_batch_autotune(hs_batch *b, const double *betas, int n_trial_sweeps) {
     float best_ms = 0.f;
     bool have = false;
     if (st == HS_OK && cudaStreamSynchronize(b->stream) != cudaSuccess) st = fail(HS_E_CUDA, "synchronise");
-    const int max_sc = b->resident_bytes <= hs::batch_resident_limit(b->precision) ? 2 : 1;
+    const int max_sc = b->resident_ok() ? 2 : 1;
     for (int sc = 0; st == HS_OK && sc <= max_sc; ++sc)
     for (int pf = 0; st == HS_OK && pf <= (sc == 2 ? 0 : 1); ++pf)
     for (int c = (sc == 2 ? b->occ : 1); st == HS_OK && c <= b->occ; ++c)
@@ -1950,7 +1978,7 @@ int hs_batch_set_layout(hs_batch *b, int ctas_per_sm, int align_rows, int prefet
     if (ctas_per_sm < 1 || ctas_per_sm > b->occ) return fail(HS_E_INVALID, "ctas_per_sm out of range");
     if (align_rows < 0 || align_rows > 2 || (prefetch != 0 && prefetch != 1) || schedule < 0 || schedule > 2)
         return fail(HS_E_INVALID, "align_rows must be 0, 1 or 2, prefetch 0 or 1, schedule 0, 1 or 2");
-    if (schedule == 2 && b->resident_bytes > hs::batch_resident_limit(b->precision))
+    if (schedule == 2 && !b->resident_ok())
         return fail(HS_E_INVALID, "the resident schedule needs every member's spins in one CTA's shared memory");
     b->prefetch = prefetch;
     b->schedule = schedule;

@@ -17,12 +17,10 @@
 #include <cuda_runtime.h>
 
 #include "batch.h"
-#include "device.cuh"
+#include "group.cuh"
 
 namespace hs {
 namespace {
-
-constexpr long long kBarrierCycles = 2000000000LL;  // about one second
 
 // Grid-wide barrier on a monotonic 64-bit arrival count (zeroed before the
 // launch): barrier k completes when the count reaches n_ctas (k + 1), so
@@ -444,6 +442,51 @@ __global__ void __launch_bounds__(kBlock, 2) batch_resident_kernel(const BatchAr
     for (uint32_t i = threadIdx.x; i < n16; i += kBlock) w16[i] = s_state[i];
 }
 
+// The resident schedule of FP64 batches with fewer members than half the SMs:
+// one cluster of several CTAs per member instead of one CTA, by the loop that
+// sweeps a single small lattice (group.cuh), its spins in L2.  One CTA per
+// member was bound by the FP64 and multiply pipes of the SMs it ran on while
+// the rest idled: 48 members of 16^3 took 39.8 us per sweep on 48 SMs.
+// kResidentRing sweeps per launch leave their sums in b.group, [member][sweep]
+// [colour][CTA][kPartials]; the fold kernel after it adds them to the members'
+// accumulators in sweep order.  (FP32 and FP16 keep one CTA per member: their
+// sums are grouped by its threads.)
+__global__ void __launch_bounds__(kClusterThreads, 1) batch_cluster_kernel(const BatchArgs b, int ctas, int s0,
+                                                                           int n_sweeps, int depth) {
+    pdl_enter();
+    const int r = (int)blockIdx.x / ctas;
+    const BatchMember &m = b.members[r];
+    PassArgs a = member_args(m, 0, m.sweep0 + (uint32_t)s0);
+    a.partials = b.group + (size_t)r * kResidentRing * 2 * ctas * kPartials;
+    a.acc = m.acc;
+    a.div_nxv = b.member_rows[r];
+    sweep_group<HS_FP64, 1, true, 0, false, false>(a, m.planes, n_sweeps, 0, depth, 0ull, (int)blockIdx.x - r * ctas,
+                                                   ctas);
+}
+
+__global__ void __launch_bounds__(kBlock) batch_group_fold_kernel(const BatchArgs b, int ctas, int s0, int n_sweeps) {
+    __shared__ double s_tot[kResidentRing][kPartials];
+    __shared__ double s_obs[kResidentRing][8];
+    pdl_enter();
+    const double *p = b.group + (size_t)blockIdx.x * kResidentRing * 2 * ctas * kPartials;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = warp; i < n_sweeps; i += kBlock / 32) {  // both colours' CTAs: at most 32 partials
+        double t[kPartials];
+#pragma unroll
+        for (int q = 0; q < kPartials; ++q)
+            t[q] = lane < 2 * ctas ? __ldcg(p + ((size_t)i * 2 * ctas + lane) * kPartials + q) : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < kPartials; ++q) t[q] += __shfl_xor_sync(0xffffffffu, t[q], o);
+        if (lane == 0)
+#pragma unroll
+            for (int q = 0; q < kPartials; ++q) s_tot[i][q] = t[q];
+    }
+    __syncthreads();
+    if (warp == 0) resident_fold(b.members[blockIdx.x], s_tot, s_obs, s0, n_sweeps, b.n_equil);
+}
+
 // Zero every member's accepted-move counter (hs_batch_run's count covers its
 // own sweeps): one launch for the whole batch.
 __global__ void batch_reset_kernel(const BatchMember *members, int n) {
@@ -615,6 +658,76 @@ cudaError_t launch_batch_resident(int precision, const BatchArgs &b, size_t smem
     case HS_FP16: return resident_p<HS_FP16>(b, smem, s);
     default: return cudaErrorInvalidValue;
     }
+}
+
+namespace {
+void cluster_launch_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int members, int ctas, int threads,
+                           cudaStream_t s) {
+    cfg.gridDim = dim3((unsigned)(members * ctas));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = held_passes(HS_FP64, threads) * pass_bytes(HS_FP64, threads);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+}
+}  // namespace
+
+// CTAs per member and their threads, by estimated time of a sweep: as many
+// rounds of clusters as the device holds at once need, each 6 us (the serial
+// chain of two passes) and the largest member's attempts at 0.18 per ns and SM.
+BatchClusters batch_cluster_plan(int precision, int n_members, int64_t max_sites, int n_sm) {
+    BatchClusters best{0, 0};
+    if (precision != HS_FP64 || max_sites > kBatchClusterSites || 2 * n_members > n_sm) return best;
+    if (cudaFuncSetAttribute(batch_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeldBytes) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(batch_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return best;
+    }
+    const int warps = (int)((max_sites / 2 + 31) / 32);
+    double best_ns = 0.0;
+    for (int c = 2; c <= 16; ++c) {
+        if (c > warps) break;
+        const int per = 32 * ((warps + c - 1) / c);
+        const int threads = per < kClusterThreads ? per : kClusterThreads;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute attr[2];
+        cluster_launch_config(cfg, attr, n_members, c, threads, nullptr);
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, batch_cluster_kernel, &cfg) != cudaSuccess || n < 1) {
+            cudaGetLastError();  // no such cluster on this device
+            continue;
+        }
+        const double ns = (double)((n_members + n - 1) / n) * (6000.0 + (double)max_sites / (0.18 * c));
+        if (best.ctas == 0 || ns < best_ns) {
+            best = BatchClusters{c, threads};
+            best_ns = ns;
+        }
+    }
+    return best;
+}
+
+size_t batch_cluster_bytes(int n_members, const BatchClusters &p) {
+    return (size_t)n_members * kResidentRing * 2 * p.ctas * kPartials * sizeof(double);
+}
+
+cudaError_t launch_batch_clusters(const BatchArgs &b, const BatchClusters &p, cudaStream_t s) {
+    for (int s0 = 0; s0 < b.n_total; s0 += kResidentRing) {
+        const int k = b.n_total - s0 < kResidentRing ? b.n_total - s0 : kResidentRing;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute attr[2];
+        cluster_launch_config(cfg, attr, b.n_members, p.ctas, p.threads, s);
+        cudaError_t e = cudaLaunchKernelEx(&cfg, batch_cluster_kernel, b, p.ctas, s0, k, held_passes(HS_FP64, p.threads));
+        if (e == cudaSuccess) e = launch_chained(batch_group_fold_kernel, b.n_members, s, b, p.ctas, s0, k);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_batch(int precision, const BatchArgs &b, int grid, cudaStream_t s, int prefetch) {

@@ -48,6 +48,8 @@ struct BatchArgs {
     int inject_skip;         // test hook: 1 = CTA 0 skips its first barrier arrival
     int zaxis_all;           // 1: every member's easy axis is (0, 0, 1): FP32 / FP16 run the S.e = S_z kernels
     int kzero_all;           // 1: besides, every member's K is +0: they run the kernels without the K term
+    double *group;           // sums of the cluster schedule's sweeps (batch_cluster_bytes)
+    const FastDiv *member_rows;  // that schedule: division by each member's Lx / 2 (one site per work item)
 };
 
 // sites per work item of a batch member: 16-byte loads for FP64 and FP32,
@@ -63,6 +65,16 @@ int batch_occupancy(int precision, int prefetch);
 // memory (smem bytes, at most batch_resident_limit(precision)) for the whole run
 cudaError_t launch_batch_resident(int precision, const BatchArgs &b, size_t smem, cudaStream_t s);
 size_t batch_resident_limit(int precision);
+// the resident schedule of FP64 batches of few members: one cluster of ctas
+// CTAs (0: none) of that many threads per member, for members of at most
+// kBatchClusterSites sites (24^3 measured 2.5 times the persistent schedule)
+constexpr int64_t kBatchClusterSites = 16384;
+struct BatchClusters {
+    int ctas, threads;
+};
+BatchClusters batch_cluster_plan(int precision, int n_members, int64_t max_sites, int n_sm);
+size_t batch_cluster_bytes(int n_members, const BatchClusters &p);
+cudaError_t launch_batch_clusters(const BatchArgs &b, const BatchClusters &p, cudaStream_t s);
 // zero every member's accepted-move counter (reads b.members on the device)
 cudaError_t launch_batch_reset(const BatchArgs &b, cudaStream_t s);
 
