@@ -31,6 +31,7 @@
 #include "cluster.h"
 #include "hs_impl.h"
 #include "slab.h"
+#include "table_group.h"
 #include "upload.h"
 
 namespace {
@@ -448,6 +449,8 @@ int configure_launch(hs_lattice *h) {
         const int occ = std::min(hs::pass_occupancy(h->precision, L, 0), hs::pass_occupancy(h->precision, L, 1));
         if (bps <= 0 || bps > occ) bps = occ;
         h->n_blocks = std::min(hs::pass_blocks(h->precision, L, h->n_sm, bps), h->max_blocks);
+        if (r.kernel == HS_KERNEL_AUTO && r.blocks_per_sm == 0 && r.prefetch == 0)
+            h->group.ctas = hs::table_group_ctas(h->precision, L, h->n_blocks, h->n_sm);
         return HS_OK;
     }
     L.vec = r.vec_width ? r.vec_width : default_vec(h);
@@ -836,9 +839,12 @@ int hs_sweep(hs_lattice *h, double beta, int64_t n_sweeps) {
         for (int64_t s = 0; s < n_sweeps;) {
             const int k = (int)std::min<int64_t>(h->fold_ring, n_sweeps - s);
             a.sweep = (uint32_t)(h->sweep + (uint64_t)s);
-            HS_CUDA(hs::launch_group(h->precision, h->L, h->group, a, k, arrivals, h->stream));
+            if (h->L.structured)
+                HS_CUDA(hs::launch_group(h->precision, h->L, h->group, a, k, arrivals, h->stream));
+            else
+                HS_CUDA(hs::launch_table_group(h->precision, h->L, a, h->group.ctas, k, arrivals, h->stream));
             HS_CUDA(hs::launch_fold(a, k, h->stream));
-            arrivals += (unsigned long long)h->group.ctas * (2 * k - 1);  // no barrier after a launch's last pass
+            arrivals += (unsigned long long)h->group.ctas * (h->L.n_colours * k - 1);  // none after the last pass
             s += k;
         }
         h->sweep += (uint64_t)n_sweeps;
@@ -1367,6 +1373,7 @@ std::vector<hs_launch> tune_candidates(hs_lattice *h) {
     std::vector<hs_launch> out;
     const Layout &L = h->L;
     if (!L.structured) {
+        out.push_back(hs_launch{});  // the automatic launch (a small lattice's is one for a whole group of sweeps)
         for (int b = 1; b <= 8; ++b)
             for (int pf : {1, 2}) out.push_back({HS_KERNEL_TABLE, 1, b, 0, pf});
         return out;

@@ -27,6 +27,7 @@
 #include <type_traits>
 
 #include "device.cuh"
+#include "table.cuh"
 
 namespace hs {
 namespace {
@@ -343,19 +344,6 @@ __global__ void __launch_bounds__(kBlock, 2) sc_march_kernel(const PassArgs a) {
     write_partials<C, MEAS>(a, acc.E(J, K), acc.X(), acc.Y(), acc.Z(), acc.n);
 }
 
-// A site's FP64 field, its neighbours read again through the table (for a decision that FP32 left open).
-__device__ __noinline__ double3 table_field64(const Vec<double, 4> *spins, const int32_t *nbr, int64_t i, int64_t n_pad,
-                                              int width) {
-    double3 h = make_double3(0.0, 0.0, 0.0);
-    for (int k = 0; k < width; ++k) {
-        const Vec<double, 4> n = spins[__ldg(nbr + (int64_t)k * n_pad + i)];
-        h.x += n.v[0];
-        h.y += n.v[1];
-        h.z += n.v[2];
-    }
-    return h;
-}
-
 // ----------------------------------------------------------------- table pass
 // One colour pass over renumbered sites [begin, end) with a neighbour table.
 // Neighbours sum in stored order; padding points at a zero dummy spin.
@@ -386,38 +374,15 @@ __global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (W > 0 ? 4 : 5)) ta
     S4 *spins = reinterpret_cast<S4 *>(a.spins4);
     C J, K, ex, ey, ez, beta;
     load_params(a, J, K, ex, ey, ez, beta);
-    C accE = C(0), accX = C(0), accY = C(0), accZ = C(0);
-    unsigned nacc = 0;
+    TableAcc<P> acc;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = a.begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.end; i += stride) {
-        C hx = C(0), hy = C(0), hz = C(0);
-        C lx = C(0), ly = C(0), lz = C(0);
-        // FP64 without the tensor: the field in FP32 (the decision's), the energy's part of it in FP64
-        constexpr bool kNarrow = P == HS_FP64 && !TEN;
-        float gx = 0.0f, gy = 0.0f, gz = 0.0f;
-        int big = 0;
+        TableField<P, MEAS, TEN> f;
         if (PFL2 && i + stride < a.end) {
             for (int k = 0; k < a.width; ++k)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(a.nbr + (int64_t)k * a.n_pad + i + stride));
             asm volatile("prefetch.global.L2 [%0];" ::"l"(spins + i + stride));
         }
-        auto add = [&](int32_t j, const S4 &n) {
-            const C nx = to_c(n.v[0]), ny = to_c(n.v[1]), nz = to_c(n.v[2]);
-            if constexpr (kNarrow) {
-                gx = f_add(gx, narrow(nx, big));
-                gy = f_add(gy, narrow(ny, big));
-                gz = f_add(gz, narrow(nz, big));
-            } else {
-                hx += nx;
-                hy += ny;
-                hz += nz;
-            }
-            if (MEAS && j < a.colour_begin) {
-                lx += nx;
-                ly += ny;
-                lz += nz;
-            }
-        };
         if constexpr (W > 0) {
             int32_t jj[W];
             S4 nn[W];
@@ -426,76 +391,19 @@ __global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (W > 0 ? 4 : 5)) ta
 #pragma unroll
             for (int k = 0; k < W; ++k) nn[k] = spins[jj[k]];
 #pragma unroll
-            for (int k = 0; k < W; ++k) add(jj[k], nn[k]);
+            for (int k = 0; k < W; ++k) f.add(a, jj[k], nn[k]);
         } else {
             for (int k = 0; k < a.width; ++k) {
                 const int32_t j = __ldg(a.nbr + (int64_t)k * a.n_pad + i);
-                add(j, spins[j]);
+                f.add(a, j, spins[j]);
             }
         }
         S4 s = spins[i];
-        C sx = to_c(s.v[0]), sy = to_c(s.v[1]), sz = to_c(s.v[2]);
-        C tx, ty, tz;
-        bool accepted;
-        if constexpr (P == HS_FP64) {
-            const uint32_t site = __ldg(a.nat + i);
-            const Trial64 t =
-                trial64(trial64_block(site, a.sweep, (uint32_t)a.colour, 0u, a.replica, a.key0, a.key1), a.sc_tab);
-            const uint4 pw = trial64_block(site, a.sweep, (uint32_t)a.colour, 1u, a.replica, a.key0, a.key1);
-            const float uf = (float)(pw.x >> 8) * 0x1p-24f;
-            tx = t.x;
-            ty = t.y;
-            tz = t.z;
-            if constexpr (kNarrow) {
-                const float fx = narrow(sx, big), fy = narrow(sy, big), fz = narrow(sz, big);
-                const Dots32<float> d = site_math32<float>(fx, fy, fz, t.fx, t.fy, t.fz, gx, gy, gz, a.fJ, a.fK,
-                                                           a.fe[0], a.fe[1], a.fe[2]);
-                int dec = decide64(-a.fbeta * d.dH, a.fdelta, uf);
-                if (big > 0x3FF00100) dec = -1;  // 1 + 2^-12: no unit vectors
-                if (dec < 0) {
-                    const double3 h = table_field64(spins, a.nbr, i, a.n_pad, a.width);
-                    dec = accept_wide<false>(sx, sy, sz, tx, ty, tz, h.x, h.y, h.z, J, K, ex, ey, ez, beta,
-                                             (double)bits53(pw.x, pw.y) * 0x1p-53, uf);
-                }
-                accepted = dec > 0;
-            } else {
-                accepted = metropolis<C, TEN>(sx, sy, sz, tx, ty, tz, hx, hy, hz, J, K, ex, ey, ez, beta,
-                                              (double)bits53(pw.x, pw.y) * 0x1p-53, uf, a.A)
-                               .acc;
-            }
-        } else {
-            float u;
-            draw_trial_rank<P>((uint32_t)(i - a.colour_begin), a.sweep, (uint32_t)a.colour, a.replica, a.key0,
-                               a.key1, tx, ty, tz, u);
-            const Dots32<float> d =
-                site_math32<float, TEN>(sx, sy, sz, tx, ty, tz, hx, hy, hz, J, K, ex, ey, ez, a.fA);
-            accepted = accept32(d.dH, u, neg_beta_log2e(beta));
-        }
-        if (accepted) {
-            sx = tx;
-            sy = ty;
-            sz = tz;
-            s.v[0] = to_store<S, C>(tx);
-            s.v[1] = to_store<S, C>(ty);
-            s.v[2] = to_store<S, C>(tz);
-            spins[i] = s;
-            ++nacc;
-        }
-        if (MEAS) {
-            const C se = sx * ex + sy * ey + sz * ez;
-            accE += -J * (sx * lx + sy * ly + sz * lz) - K * se * se;
-            if constexpr (TEN) {
-                if constexpr (P == HS_FP64)
-                    accE -= quad64(sx, sy, sz, a.A);
-                else
-                    accE -= quad32<float>(sx, sy, sz, a.fA);
-            }
-            accX += sx;
-            accY += sy;
-            accZ += sz;
-        }
+        TableTrial<P> t;
+        draw_table_trial<P>(a, i, t);
+        if (table_update<P, MEAS, TEN>(a, i, spins, f, t, s, J, K, ex, ey, ez, beta, acc)) spins[i] = s;
     }
-    write_partials<C, MEAS>(a, accE, accX, accY, accZ, nacc);
+    write_partials<C, MEAS>(a, acc.e, acc.x, acc.y, acc.z, acc.n);
 }
 
 // ----------------------------------------------------------------- measure

@@ -1,0 +1,23 @@
+// Sweeps of a small neighbour-table lattice, a group of them in one launch (table_group.cu).
+#pragma once
+
+#include "hs_impl.h"
+
+namespace hs {
+
+// The largest table lattices that sweep this way.
+constexpr int64_t kTableGroupSites = 600000;
+
+// Renumbered sites of colour class c: begin[c] .. begin[c + 1] - 1.
+struct TableClasses {
+    int64_t begin[65];
+};
+
+// CTAs of the launch (the launch chain's n_blocks), or 0 where it does not
+// apply: the tensor term, widths other than 6, 8 and 12, larger lattices, or a
+// grid that is not resident at once.
+int table_group_ctas(int precision, const Layout &L, int n_blocks, int n_sm);
+cudaError_t launch_table_group(int precision, const Layout &L, const PassArgs &a, int ctas, int n_sweeps,
+                               unsigned long long arrivals, cudaStream_t s);
+
+}  // namespace hs

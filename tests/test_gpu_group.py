@@ -44,3 +44,40 @@ def test_group_equals_the_launch_chain(precision, dims, e, K, tensor, meas):
     np.testing.assert_array_equal(got[0], want[0])
     assert got[2:] == want[2:]
     np.testing.assert_allclose(got[1], want[1], rtol=0, atol=1e-12 * max(1.0, np.abs(want[1]).max()))
+
+
+def _table(kind, precision, chain, sweeps, meas):
+    from paper_2106_11286_gb300 import inputs
+    kw = dict(precision=precision, seed=7, K=0.2, e=(1, 1, 1))
+    if kind == "csr":
+        rp, col, mask = inputs.bcc_nanoparticle(radius=9.3, box=22, vacancy_fraction=0.05, seed=3)
+        lat = hs.Lattice("csr", row_ptr=rp, col_idx=col, site_mask=mask, **kw)
+    elif kind == "sc_open":
+        lat = hs.Lattice("sc", dims=(31, 17, 23), periodic=False, **kw)
+    elif kind == "fcc_masked":
+        lat = hs.Lattice("fcc", dims=(7, 5, 9), site_mask=inputs.vacancy_mask(7 * 5 * 9 * 4, 0.1, 5), **kw)
+    elif kind == "bcc_large":
+        lat = hs.Lattice("bcc", dims=(60, 56, 50), **kw)
+    else:
+        lat = hs.Lattice("bcc", dims=(2, 2, 1), **kw)
+    with lat:
+        if chain:
+            lat.set_launch(kernel="table", blocks_per_sm=8)
+        lat.init()
+        lat.accumulate(meas)
+        for n in sweeps:
+            lat.sweep(0.9, n)
+        moments, count = lat.read_accumulator()
+        return lat.get_spins(), moments, count, lat.measure()["accept_rate"], lat.info.sweep
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("kind", ["csr", "sc_open", "fcc_masked", "bcc_large", "bcc_tiny"])
+@pytest.mark.parametrize("meas", [True, False])
+def test_table_group_equals_the_launch_chain(precision, kind, meas):
+    """The neighbour-table lattices' group launch, likewise (widths 8, 6, 12; greedy classes; vacancies)."""
+    sweeps = (3, 1) if kind == "bcc_large" else (66, 1)
+    got, want = (_table(kind, precision, chain, sweeps, meas) for chain in (False, True))
+    np.testing.assert_array_equal(got[0], want[0])
+    assert got[2:] == want[2:]
+    np.testing.assert_allclose(got[1], want[1], rtol=0, atol=1e-12 * max(1.0, np.abs(want[1]).max()))
