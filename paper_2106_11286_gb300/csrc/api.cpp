@@ -449,8 +449,11 @@ int configure_launch(hs_lattice *h) {
         const int occ = std::min(hs::pass_occupancy(h->precision, L, 0), hs::pass_occupancy(h->precision, L, 1));
         if (bps <= 0 || bps > occ) bps = occ;
         h->n_blocks = std::min(hs::pass_blocks(h->precision, L, h->n_sm, bps), h->max_blocks);
-        if (r.kernel == HS_KERNEL_AUTO && r.blocks_per_sm == 0 && r.prefetch == 0)
-            h->group.ctas = hs::table_group_ctas(h->precision, L, h->n_blocks, h->n_sm);
+        if (r.kernel == HS_KERNEL_AUTO && r.blocks_per_sm == 0 && r.prefetch == 0) {
+            const hs::TableGroupPlan p = hs::table_group_plan(h->precision, L, h->n_blocks, h->n_sm);
+            h->group.ctas = p.ctas;
+            h->group.threads = p.threads;
+        }
         return HS_OK;
     }
     L.vec = r.vec_width ? r.vec_width : default_vec(h);
@@ -842,7 +845,8 @@ int hs_sweep(hs_lattice *h, double beta, int64_t n_sweeps) {
             if (h->L.structured)
                 HS_CUDA(hs::launch_group(h->precision, h->L, h->group, a, k, arrivals, h->stream));
             else
-                HS_CUDA(hs::launch_table_group(h->precision, h->L, a, h->group.ctas, k, arrivals, h->stream));
+                HS_CUDA(hs::launch_table_group(h->precision, h->L, a, {h->group.ctas, h->group.threads}, k, arrivals,
+                                               h->stream));
             HS_CUDA(hs::launch_fold(a, k, h->stream));
             arrivals += (unsigned long long)h->group.ctas * (h->L.n_colours * k - 1);  // none after the last pass
             s += k;

@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include "batch.h"
+#include "fit_cache.h"
 #include "group.cuh"
 
 namespace hs {
@@ -695,15 +696,17 @@ BatchClusters batch_cluster_plan(int precision, int n_members, int64_t max_sites
         if (c > warps) break;
         const int per = 32 * ((warps + c - 1) / c);
         const int threads = per < kClusterThreads ? per : kClusterThreads;
-        cudaLaunchConfig_t cfg{};
-        cudaLaunchAttribute attr[2];
-        cluster_launch_config(cfg, attr, n_members, c, threads, nullptr);
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, batch_cluster_kernel, &cfg) != cudaSuccess || n < 1) {
+        const int n = cached_fit((const void *)batch_cluster_kernel, c, threads, [&] {
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute attr[2];
+            cluster_launch_config(cfg, attr, 1, c, threads, nullptr);
+            cfg.numAttrs = 1;
+            int most = 0;
+            if (cudaOccupancyMaxActiveClusters(&most, batch_cluster_kernel, &cfg) == cudaSuccess) return most;
             cudaGetLastError();  // no such cluster on this device
-            continue;
-        }
+            return 0;
+        });
+        if (n < 1) continue;
         const double ns = (double)((n_members + n - 1) / n) * (6000.0 + (double)max_sites / (0.18 * c));
         if (best.ctas == 0 || ns < best_ns) {
             best = BatchClusters{c, threads};

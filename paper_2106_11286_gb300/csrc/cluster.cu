@@ -16,19 +16,20 @@
 // travel, and the sums of several passes are kept in shared memory and reduced
 // together, independent chains side by side.  us per sweep, this launch and
 // the launch chain: 16^3 FP64 6.0 and 15.6, 16^3 FP32 4.2 and 6.7, 24^3 FP32 4.3
-// and 6.8, 32^3 FP32 5.1 and 6.9.
+// and 6.8.
 //
 // Lattices of up to kGridSites sites run the same loop on the whole device as
 // one cooperative launch, with a barrier over the grid: it takes about as long
 // as the cluster's plus one atomic and one poll, still less than ending a
-// launch and starting the next: 64^3 FP32 5.6 and 8.6 us per sweep, 96^3 10.0
-// and 11.9, 128^3 15.9 and 18.3, 160^3 27.4 and 27.6; FP64 32^3 8.9 and 16.7,
-// 64^3 20.7 and 26.2, 96^3 46.2 and 48.4, 128^3 94.0 and 92.3.
+// launch and starting the next: 64^3 FP32 5.4 and 8.6 us per sweep, 96^3 10.0
+// and 11.9, 128^3 15.9 and 18.3, 160^3 27.4 and 27.6; FP64 32^3 7.2 and 16.7,
+// 64^3 20.5 and 26.2, 96^3 46.2 and 48.4, 128^3 94.0 and 92.3.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
 #include "cluster.h"
+#include "fit_cache.h"
 #include "group.cuh"
 
 namespace hs {
@@ -104,32 +105,34 @@ void group_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int p
     cfg.numAttrs = 2;
 }
 
+// The device takes kernel k as p asks.
+bool ask_fits(int precision, const GroupPlan &p, const void *k, int n_sm) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[2];
+    group_config(cfg, attr, precision, p, nullptr);
+    int n = 0;
+    bool ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeldBytes) == cudaSuccess;
+    if (ok && p.grid) {
+        ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, p.threads, cfg.dynamicSmemBytes) == cudaSuccess &&
+             n * n_sm >= p.ctas;
+    } else if (ok) {
+        cfg.numAttrs = 1;
+        ok = (p.ctas <= 8 || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+             cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n >= 1;
+    }
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+
 // Both variants (with and without the fused measurement) fit the device as p asks.
 bool plan_fits(int precision, const GroupPlan &p, bool ten, bool ax, int n_sm) {
     for (int meas = 0; meas < 2; ++meas) {
         const void *k = group_kernel(precision, p, meas != 0, ten, ax);
-        cudaLaunchConfig_t cfg{};
-        cudaLaunchAttribute attr[2];
-        group_config(cfg, attr, precision, p, nullptr);
-        int n = 0;
-        bool ok = k && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeldBytes) == cudaSuccess;
-        if (ok && p.grid) {
-            ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, p.threads, cfg.dynamicSmemBytes) == cudaSuccess &&
-                 n * n_sm >= p.ctas;
-        } else if (ok) {
-            cfg.numAttrs = 1;
-            ok = (p.ctas <= 8 ||
-                  cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
-                 cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n >= 1;
-        }
-        if (!ok) {
-            cudaGetLastError();
+        if (!k || cached_fit(k, p.ctas, p.threads, [&] { return ask_fits(precision, p, k, n_sm) ? 1 : 0; }) == 0)
             return false;
-        }
     }
     return true;
 }
-
 }  // namespace
 
 GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, int n_sm) {
@@ -153,6 +156,7 @@ GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, in
         p.vec = 1;
         p.ctas = (int)((L.n_sites / 2 + kBlock - 1) / kBlock);
     }
+    spread_ctas(L.n_sites / 2 / p.vec, n_sm, p.ctas, p.threads);
     return plan_fits(precision, p, ten, ax, n_sm) ? p : none;
 }
 

@@ -6,11 +6,11 @@
 namespace hs {
 
 // The largest lattices that run in one cluster: beyond them its 16 SMs take
-// longer over a pass than a barrier over the whole device costs (FP32 40^3: 7.5
-// us per sweep in the cluster, 5.5 on the grid; FP64 24^3: 10.4 against 8.9 for
-// 32^3 on the grid).
-constexpr int64_t kClusterSites = 32768;   // FP32, FP16
-constexpr int64_t kClusterSites64 = 8192;  // FP64
+// longer over a pass than a barrier over the whole device costs (us per sweep
+// FP32: 24^3 4.3 in the cluster, 32^3 5.1 there, 40^3 5.0 on the grid; FP64 16^3
+// 6.0 and 20^3 7.9 in the cluster, 24^3 7.2 on the grid).
+constexpr int64_t kClusterSites = 24000;   // FP32, FP16
+constexpr int64_t kClusterSites64 = 5000;  // FP64
 // The largest that run as one cooperative launch: beyond them the launches
 // are a small part of a pass (times in cluster.cu).
 constexpr int64_t kGridSites = 3000000;    // FP32, FP16

@@ -163,6 +163,18 @@ inline float decision_band(double beta, double J, double K, int width) {
     return (float)(beta * (aJ * (width > 6 ? 6e-5 : 2e-5) + aK * 1e-5) * 1.001);
 }
 
+// Fewer items than the SMs have threads of one CTA each: CTAs of as few warps
+// as spread them over every SM (a pass of few warps is bound by each SM's
+// multiply and FP64 pipes and its load latency; the warps' items, and with them
+// the FP32 sums, stay the same).  us per sweep with CTAs of 256 threads and so:
+// FP64 32^3 8.9 and 7.2, fcc FP64 of 73,656 sites 26.3 and 20.6; 48^3 FP32 5.6
+// and 5.0.
+inline void spread_ctas(int64_t items, int n_sm, int &ctas, int &threads) {
+    if (items >= (int64_t)n_sm * kBlock) return;
+    threads = 32 * (int)((items + 32 * (int64_t)n_sm - 1) / (32 * (int64_t)n_sm));
+    ctas = (int)((items + threads - 1) / threads);
+}
+
 size_t storage_size(int precision);
 
 // Record the thread-local message returned by hs_last_error; returns code.

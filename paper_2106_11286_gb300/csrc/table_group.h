@@ -13,11 +13,14 @@ struct TableClasses {
     int64_t begin[65];
 };
 
-// CTAs of the launch (the launch chain's n_blocks), or 0 where it does not
-// apply: the tensor term, widths other than 6, 8 and 12, larger lattices, or a
-// grid that is not resident at once.
-int table_group_ctas(int precision, const Layout &L, int n_blocks, int n_sm);
-cudaError_t launch_table_group(int precision, const Layout &L, const PassArgs &a, int ctas, int n_sweeps,
-                               unsigned long long arrivals, cudaStream_t s);
+// CTAs of the launch and their threads (the launch chain's n_blocks of kBlock,
+// or spread_ctas), ctas 0 where it does not apply: the tensor term, widths
+// other than 6, 8 and 12, larger lattices, or a grid not resident at once.
+struct TableGroupPlan {
+    int ctas, threads;
+};
+TableGroupPlan table_group_plan(int precision, const Layout &L, int n_blocks, int n_sm);
+cudaError_t launch_table_group(int precision, const Layout &L, const PassArgs &a, const TableGroupPlan &p,
+                               int n_sweeps, unsigned long long arrivals, cudaStream_t s);
 
 }  // namespace hs
