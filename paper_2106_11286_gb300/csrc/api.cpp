@@ -208,7 +208,7 @@ struct hs_lattice {
     Layout L{};
     int n_blocks = 1;
     hs_launch req{};        // requested launch configuration (0 = automatic)
-    hs::GroupPlan group{0, 0, 1, false};  // small lattices' automatic launch: a whole group of sweeps at once
+    hs::GroupPlan group{0, 0, 1, hs::kGroupCluster, 0, 0};  // small lattices' automatic launch: a whole group of sweeps at once
     int max_blocks = 1;     // capacity of the partials buffer
     int fold_ring = 1;      // sweeps per ring fold (slot sets of the partials buffer)
     double *partials = nullptr;
@@ -437,7 +437,7 @@ int configure_launch(hs_lattice *h) {
         return fail(HS_E_INVALID, "a slab's sweep is in progress");
     const hs_launch &r = h->req;
     L.tensor = h->tensor;
-    h->group = hs::GroupPlan{0, 0, 1, false};
+    h->group = hs::GroupPlan{0, 0, 1, hs::kGroupCluster, 0, 0};
     if (!L.structured) {
         L.kernel = hs::kTable;
         // request 1 = L2 prefetch of the next site's table row, 2 = off, 0 = automatic (on for FP32 tables of

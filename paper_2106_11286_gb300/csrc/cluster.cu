@@ -43,6 +43,14 @@ __global__ void __launch_bounds__(kClusterThreads, 1) sc_cluster_kernel(const Pa
                                               (int)gridDim.x);
 }
 
+template <int P, int V, bool MEAS, int AX>
+__global__ void __launch_bounds__(kClusterThreads, 1) sc_slab_kernel(const PassArgs args, void *planes, int n_sweeps,
+                                                                     int alternate, int depth) {
+    pdl_enter();
+    (void)alternate;  // a warp's items and their sum are the same in either direction
+    sweep_slabs<P, V, MEAS, AX>(args, planes, n_sweeps, depth, (int)blockIdx.x, (int)gridDim.x);
+}
+
 template <int P, int V, bool MEAS, int AX, bool TEN>
 __global__ void __launch_bounds__(kBlock, 2) sc_grid_kernel(const PassArgs args, void *planes, int n_sweeps,
                                                             int alternate, int depth, unsigned long long arrivals) {
@@ -52,7 +60,13 @@ __global__ void __launch_bounds__(kBlock, 2) sc_grid_kernel(const PassArgs args,
 
 // The variants of one precision and width: the tensor term, or FP32's S.e = S_z.
 template <int P, int V, bool MEAS>
-const void *group_ptr(bool grid, bool ten, bool ax) {
+const void *group_ptr(GroupKind kind, bool ten, bool ax) {
+    const bool grid = kind == kGroupGrid;
+    if (kind == kGroupSlabs) {
+        if constexpr (P == HS_FP32)
+            if (ax) return (const void *)sc_slab_kernel<P, V, MEAS, 1>;
+        return (const void *)sc_slab_kernel<P, V, MEAS, 0>;
+    }
     if (ten)
         return grid ? (const void *)sc_grid_kernel<P, V, MEAS, 0, true> : (const void *)sc_cluster_kernel<P, V, MEAS, 0, true>;
     if constexpr (P == HS_FP32)
@@ -63,7 +77,7 @@ const void *group_ptr(bool grid, bool ten, bool ax) {
 }
 
 template <int P>
-const void *group_vec(int vec, bool meas, bool grid, bool ten, bool ax) {
+const void *group_vec(int vec, bool meas, GroupKind grid, bool ten, bool ax) {
     switch (vec) {
     case 1: return meas ? group_ptr<P, 1, true>(grid, ten, ax) : group_ptr<P, 1, false>(grid, ten, ax);
     case 2: return meas ? group_ptr<P, 2, true>(grid, ten, ax) : group_ptr<P, 2, false>(grid, ten, ax);
@@ -77,9 +91,9 @@ const void *group_vec(int vec, bool meas, bool grid, bool ten, bool ax) {
 
 const void *group_kernel(int precision, const GroupPlan &p, bool meas, bool ten, bool ax) {
     switch (precision) {
-    case HS_FP64: return group_vec<HS_FP64>(p.vec, meas, p.grid, ten, ax);
-    case HS_FP32: return group_vec<HS_FP32>(p.vec, meas, p.grid, ten, ax);
-    case HS_FP16: return group_vec<HS_FP16>(p.vec, meas, p.grid, ten, ax);
+    case HS_FP64: return group_vec<HS_FP64>(p.vec, meas, p.kind, ten, ax);
+    case HS_FP32: return group_vec<HS_FP32>(p.vec, meas, p.kind, ten, ax);
+    case HS_FP16: return group_vec<HS_FP16>(p.vec, meas, p.kind, ten, ax);
     default: return nullptr;
     }
 }
@@ -88,10 +102,10 @@ void group_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int p
                   cudaStream_t s) {
     cfg.gridDim = dim3((unsigned)p.ctas);
     cfg.blockDim = dim3((unsigned)p.threads);
-    cfg.dynamicSmemBytes = held_passes(precision, p.threads) * pass_bytes(precision, p.threads);
+    cfg.dynamicSmemBytes = p.smem + p.depth * pass_bytes(precision, p.threads);
     cfg.stream = s;
     cfg.attrs = attr;
-    if (p.grid) {
+    if (p.kind == kGroupGrid) {
         attr[0].id = cudaLaunchAttributeCooperative;
         attr[0].val.cooperative = 1;
         cfg.numAttrs = 1;
@@ -111,8 +125,9 @@ bool ask_fits(int precision, const GroupPlan &p, const void *k, int n_sm) {
     cudaLaunchAttribute attr[2];
     group_config(cfg, attr, precision, p, nullptr);
     int n = 0;
-    bool ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeldBytes) == cudaSuccess;
-    if (ok && p.grid) {
+    bool ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)(p.kind == kGroupSlabs ? kSlabBytes : kHeldBytes)) == cudaSuccess;
+    if (ok && p.kind == kGroupGrid) {
         ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, p.threads, cfg.dynamicSmemBytes) == cudaSuccess &&
              n * n_sm >= p.ctas;
     } else if (ok) {
@@ -128,35 +143,62 @@ bool ask_fits(int precision, const GroupPlan &p, const void *k, int n_sm) {
 bool plan_fits(int precision, const GroupPlan &p, bool ten, bool ax, int n_sm) {
     for (int meas = 0; meas < 2; ++meas) {
         const void *k = group_kernel(precision, p, meas != 0, ten, ax);
-        if (!k || cached_fit(k, p.ctas, p.threads, [&] { return ask_fits(precision, p, k, n_sm) ? 1 : 0; }) == 0)
+        if (!k || cached_fit(k, p.ctas, p.threads + (int)(p.smem / 1024) * 1024, [&] { return ask_fits(precision, p, k, n_sm) ? 1 : 0; }) == 0)
             return false;
     }
     return true;
 }
 }  // namespace
 
+namespace {
+// The cluster whose CTAs keep a slab each in shared memory, or ctas 0: at
+// least 8 planes, and for FP32 / FP16 equal slabs of whole warps of items.
+GroupPlan slab_plan(int precision, const Layout &L, bool ax, int n_sm) {
+    const int vec = precision == HS_FP64 ? 1 : L.vec;  // FP64: one site a thread, the shortest chain
+    for (int c = std::min(16, L.Lz); c >= 8; --c) {
+        const int most = slab_planes(L.Lz, c);
+        const int64_t items = (int64_t)most * L.Ly * (L.Lh / vec);
+        if (precision != HS_FP64 && (L.Lz % c != 0 || items % 32 != 0)) continue;
+        GroupPlan p{c, (int)std::min<int64_t>(kClusterThreads, (items + 31) / 32 * 32), vec, kGroupSlabs, 0, 0};
+        p.smem = slab_bytes(storage_size(precision), L.Lz, L.Ly, L.Lh, c);
+        if (p.smem + pass_bytes(precision, p.threads) > kSlabBytes) continue;
+        p.depth = (int)std::min<size_t>(held_passes(precision, p.threads),
+                                        (kSlabBytes - p.smem) / pass_bytes(precision, p.threads));
+        if (plan_fits(precision, p, false, ax, n_sm)) return p;
+    }
+    return GroupPlan{0, 0, L.vec, kGroupCluster, 0, 0};
+}
+}  // namespace
+
 GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, int n_sm) {
-    const GroupPlan none{0, 0, L.vec, false};
-    if (!L.structured || L.slab || L.vec > 4 || L.n_sites > (precision == HS_FP64 ? kGridSites64 : kGridSites)) return none;
+    const GroupPlan none{0, 0, L.vec, kGroupCluster, 0, 0};
+    const bool wide = precision == HS_FP64;
+    if (!L.structured || L.slab || L.vec > 4 || L.n_sites > (wide ? kGridSites64 : kGridSites)) return none;
     const bool ten = L.tensor != 0, ax = zaxis != 0;
-    if (L.n_sites <= (precision == HS_FP64 ? kClusterSites64 : kClusterSites)) {
+    if (!ten && L.n_sites <= (wide ? kSlabSites64 : kSlabSites)) {
+        const GroupPlan p = slab_plan(precision, L, ax, n_sm);
+        if (p.ctas > 0) return p;
+    }
+    if (L.n_sites <= (wide ? kClusterSites64 : kClusterSites)) {
         GroupPlan p = none;
-        if (precision == HS_FP64) p.vec = 1;  // one site a thread: the shortest chain
+        if (wide) p.vec = 1;
         const int warps = (int)((L.n_sites / 2 / p.vec + 31) / 32);
         // the largest cluster that the device schedules and the warps fill
         for (p.ctas = 16; p.ctas >= 1; p.ctas /= 2) {
             if (p.ctas > warps && p.ctas > 1) continue;
             p.threads = std::min(kClusterThreads, 32 * ((warps + p.ctas - 1) / p.ctas));
+            p.depth = held_passes(precision, p.threads);
             if (plan_fits(precision, p, ten, ax, n_sm)) return p;
         }
         return none;
     }
-    GroupPlan p{n_blocks, kBlock, L.vec, true};  // FP32 / FP16: the launch chain's grid, so the same sums
-    if (precision == HS_FP64 && L.n_sites / 2 <= (int64_t)n_sm * 2 * kBlock) {  // one site a thread while they last
+    GroupPlan p{n_blocks, kBlock, L.vec, kGroupGrid, 0, 0};  // FP32 / FP16: the launch chain's grid, so the same sums
+    if (wide && L.n_sites / 2 <= (int64_t)n_sm * 2 * kBlock) {  // one site a thread while they last
         p.vec = 1;
         p.ctas = (int)((L.n_sites / 2 + kBlock - 1) / kBlock);
     }
     spread_ctas(L.n_sites / 2 / p.vec, n_sm, p.ctas, p.threads);
+    p.depth = held_passes(precision, p.threads);
     return plan_fits(precision, p, ten, ax, n_sm) ? p : none;
 }
 
@@ -171,7 +213,7 @@ cudaError_t launch_group(int precision, const Layout &L, const GroupPlan &p, con
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[2];
     group_config(cfg, attr, precision, p, s);
-    int depth = held_passes(precision, p.threads);
+    int depth = p.depth;
     void *params[] = {&args, &planes, &n_sweeps, &alternate, &depth, &arrivals};  // a cluster's kernel takes the first five
     return cudaLaunchKernelExC(&cfg, k, params);
 }

@@ -16,11 +16,19 @@ constexpr int64_t kClusterSites64 = 5000;  // FP64
 constexpr int64_t kGridSites = 3000000;    // FP32, FP16
 constexpr int64_t kGridSites64 = 1000000;  // FP64
 
-// CTAs (0: the launch chain instead) of how many threads, sites per work item;
-// grid: a cooperative launch, else one cluster.
+// The largest that keep their spins in a cluster's shared memory.
+constexpr int64_t kSlabSites = 50000;   // FP32, FP16 (16^3 2.8 against 4.2, 32^3 4.2 against 5.1, 36^3 4.4 against 5.0)
+constexpr int64_t kSlabSites64 = 5000;  // FP64 (16^3 5.2 us per sweep against 6.0 with its spins in L2, 20^3 9.6 against 7.2 on the grid)
+
+// CTAs (0: the launch chain instead) of how many threads, sites per work item,
+// and how they run: one cluster with the spins in its shared memory or in L2,
+// or a cooperative launch; bytes of the slab, passes whose sums a CTA holds.
+enum GroupKind { kGroupCluster = 0, kGroupSlabs = 1, kGroupGrid = 2 };
 struct GroupPlan {
     int ctas, threads, vec;
-    bool grid;
+    GroupKind kind;
+    size_t smem;
+    int depth;
 };
 GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, int n_sm);
 

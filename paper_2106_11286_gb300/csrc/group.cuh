@@ -247,12 +247,199 @@ __device__ __forceinline__ void sweep_group(const PassArgs &args, void *planes, 
     if constexpr (!GRID) hold(pass);
 }
 
+// Store a vector into the same shared-memory place of CTA `rank` of the cluster.
+template <typename VT>
+__device__ __forceinline__ void store_remote(uint32_t local, uint32_t rank, const VT &v) {
+    uint32_t addr;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(local), "r"(rank));
+    if constexpr (sizeof(VT) == 16) {
+        uint4 w;
+        memcpy(&w, &v, 16);
+        asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w.x), "r"(w.y), "r"(w.z),
+                     "r"(w.w)
+                     : "memory");
+    } else if constexpr (sizeof(VT) == 8) {
+        uint2 w;
+        memcpy(&w, &v, 8);
+        asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(w.x), "r"(w.y) : "memory");
+    } else if constexpr (sizeof(VT) == 4) {
+        uint32_t w;
+        memcpy(&w, &v, 4);
+        asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(w) : "memory");
+    } else {
+        unsigned short w;
+        memcpy(&w, &v, 2);
+        asm volatile("st.shared::cluster.b16 [%0], %1;" ::"r"(addr), "h"(w) : "memory");
+    }
+}
+
+// Planes of the fullest slab when Lz planes are dealt to ctas CTAs: CTA k owns
+// planes Lz k / ctas .. Lz (k + 1) / ctas - 1.
+__host__ __device__ inline int slab_planes(int Lz, int ctas) { return (Lz + ctas - 1) / ctas; }
+
+// n_sweeps sweeps of one lattice by a cluster whose CTAs keep a z-slab each in
+// shared memory, with a halo plane below and above: a pass loads from the
+// CTA's own memory (30 cycles, against the 800 of L2) and stores an accepted
+// spin of a boundary plane into the neighbour's halo as well, which the
+// barrier's release waits for without a way to L2 (sweep_group took 2.8 us a
+// pass of 16^3 FP64, of which its loads and its release were 1.0).
+// FP32 / FP16: every slab must start at a multiple of 32 items, so that the
+// warps' items are the launch chain's (see PassSums).
+// The sums of sweep_group, held and reduced alike.
+template <int P, int V, bool MEAS, int AX>
+__device__ __forceinline__ void sweep_slabs(const PassArgs &args, void *planes, int n_sweeps, int depth, int cta,
+                                            int ctas) {
+    using S = typename Tr<P>::S;
+    using C = typename Tr<P>::C;
+    using VT = Vec<S, V>;
+    extern __shared__ __align__(16) unsigned char cluster_smem[];
+    PassArgs a = args;
+    const int Lz = args.Lz;
+    const int z0 = Lz * cta / ctas, nz = Lz * (cta + 1) / ctas - z0, most = slab_planes(Lz, ctas);
+    const int below = cta == 0 ? ctas - 1 : cta - 1, above = cta == ctas - 1 ? 0 : cta + 1;
+    const int nz_below = Lz * (below + 1) / ctas - Lz * below / ctas;
+    const uint32_t row_plane = (uint32_t)a.Ly * a.Lh;           // elements of one z plane of one component
+    const uint32_t comp = (uint32_t)(most + 2) * row_plane;     // of one component's slab with its halos
+    const size_t plane = (size_t)Lz * row_plane;                // of one component in device memory
+    S *const st = reinterpret_cast<S *>(cluster_smem);
+    PassSums held;
+    held.warps = (int)blockDim.x / 32;
+    held.units = P == HS_FP64 ? (int)blockDim.x : held.warps;
+    held.depth = depth;
+    held.cta = cta;
+    held.ctas = ctas;
+    held.v = reinterpret_cast<double *>(cluster_smem + ((size_t)6 * comp * sizeof(S) + 15) / 16 * 16);
+    held.n = reinterpret_cast<unsigned *>(held.v + (size_t)depth * 4 * held.units);
+    S *const dev = static_cast<S *>(planes);
+    // the slab and its halos, array plane z holding lattice plane z0 + z - 1
+    for (uint32_t k = threadIdx.x; k < (uint32_t)(nz + 2) * row_plane; k += blockDim.x) {
+        const int z = z0 + (int)(k / row_plane) - 1;
+        const size_t from = (size_t)(z < 0 ? Lz - 1 : (z >= Lz ? 0 : z)) * row_plane + k % row_plane;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) st[q * comp + k] = dev[q * plane + from];
+    }
+    a.Lz = most + 2;
+    a.zpar = (z0 - 1) & 1;
+    a.site_off = (uint32_t)((int64_t)(z0 - 1) * a.Ly * a.Lx);
+    a.rank_off = (uint32_t)((int64_t)(z0 - 1) * row_plane);
+    const uint32_t nxv = a.Lh / V;
+    const uint32_t own_items = (uint32_t)nz * a.Ly * nxv;
+    const int rounds = (int)(((uint32_t)most * a.Ly * nxv + blockDim.x - 1) / blockDim.x);  // the same for all CTAs
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t st_addr = (uint32_t)__cvta_generic_to_shared(st);
+    C J, K, ex, ey, ez, beta;
+    load_params(a, J, K, ex, ey, ez, beta);
+    double sum[4] = {0.0, 0.0, 0.0, 0.0};
+    unsigned n = 0;
+    SiteAcc<P> acc;
+    int used = 0;
+    auto hold = [&](int pass) {
+        if constexpr (P == HS_FP64) {
+            n = acc.n;
+            sum[0] = acc.E(J, K);
+            sum[1] = acc.X();
+            sum[2] = acc.Y();
+            sum[3] = acc.Z();
+            acc = SiteAcc<P>();
+        }
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (P == HS_FP64 || lane == 0) {
+            const int u = P == HS_FP64 ? (int)threadIdx.x : warp;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) held.v[(used * 4 + q) * held.units + u] = sum[q];
+        }
+        if (lane == 0) held.n[used * held.warps + warp] = n;
+        sum[0] = sum[1] = sum[2] = sum[3] = 0.0;
+        n = 0;
+        if (++used == depth || pass == 2 * n_sweeps - 1) {
+            reduce_held<P>(a, held, used, pass);
+            used = 0;
+        }
+    };
+    cluster_arrive();  // every slab is loaded before a neighbour writes its halos
+    cluster_wait();
+    int pass = 0, round = 0;
+    bool pending = false;
+    while (true) {
+        const int c = pass & 1;
+        const uint32_t t = threadIdx.x + (uint32_t)round * blockDim.x;
+        const bool mine = t < own_items;
+        a.sweep = args.sweep + (uint32_t)(pass >> 1);
+        a.colour = c;
+        const uint32_t row = a.div_nxv.div(mine ? t : 0u);
+        const uint32_t zl = a.div_ly.div(row) + 1u;
+        const ItemOffsets f = item_offsets<V>(a, row - (zl - 1u) * a.Ly, zl, (mine ? t : 0u) - row * nxv);
+        Trials<P, V> pre;
+        if (mine) draw_trials<P, V>(a, c, f.site0, f.rank0, pre);
+        if (pending) {
+            cluster_arrive();
+            hold(pass - 1);
+            cluster_wait();
+            pending = false;
+        }
+        if (mine) {
+            const S *own[3], *oth[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                own[q] = st + (3 * c + q) * comp;
+                oth[q] = st + (3 * (1 - c) + q) * comp;
+            }
+            const S *const(&own_c)[3] = reinterpret_cast<const S *const(&)[3]>(own);
+            const S *const(&oth_c)[3] = reinterpret_cast<const S *const(&)[3]>(oth);
+            StencilItem<P, V> it;
+            load_item_from<P, V>(f, own_c, oth_c, it);
+            typename ItemField<P, V>::T h;
+            fields_of<P, V, MEAS, false>(it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, c, h);
+            if (update_item_h<P, V, MEAS, false, AX, false, true>(it.s, h, it.site0, it.rank0, c, a, J, K, ex, ey, ez,
+                                                                  beta, acc, oth_c, it.b0, &pre)) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const uint32_t at = (uint32_t)(3 * c + q) * comp + it.b0;
+                    *reinterpret_cast<VT *>(st + at) = it.s[q];
+                    // array plane 1 is the halo above the slab below, plane nz the halo below the slab above
+                    if (zl == 1u)
+                        store_remote(st_addr + (at + (uint32_t)nz_below * row_plane) * (uint32_t)sizeof(S), below,
+                                     it.s[q]);
+                    if (zl == (uint32_t)nz)
+                        store_remote(st_addr + (at - (uint32_t)nz * row_plane) * (uint32_t)sizeof(S), above, it.s[q]);
+                }
+            }
+        }
+        if constexpr (P != HS_FP64) {
+            if (MEAS) {
+                sum[0] += (double)warp_sum(acc.E(J, K));
+                sum[1] += (double)warp_sum(acc.X());
+                sum[2] += (double)warp_sum(acc.Y());
+                sum[3] += (double)warp_sum(acc.Z());
+            }
+            n += acc.n;
+            acc = SiteAcc<P>();
+        }
+        if (++round < rounds) continue;
+        round = 0;
+        if (pass == 2 * n_sweeps - 1) break;
+        ++pass;
+        pending = true;
+    }
+    hold(pass);
+    cluster_arrive();  // no CTA ends while a neighbour may still write into its shared memory
+    cluster_wait();
+    for (uint32_t k = threadIdx.x; k < (uint32_t)nz * row_plane; k += blockDim.x)
+#pragma unroll
+        for (int q = 0; q < 6; ++q) dev[q * plane + (size_t)z0 * row_plane + k] = st[q * comp + row_plane + k];
+}
+
 // Passes whose sums a CTA holds (16, or what fits in 96 KB), and the bytes of one pass.
 inline size_t pass_bytes(int precision, int threads) {
     const int units = precision == HS_FP64 ? threads : threads / 32;
     return 4 * units * sizeof(double) + threads / 32 * sizeof(unsigned);
 }
 constexpr size_t kHeldBytes = 96 * 1024;
+// shared memory of a CTA that keeps its slab there (sweep_slabs), before its held sums
+inline size_t slab_bytes(size_t elem, int Lz, int Ly, int Lh, int ctas) {
+    return ((size_t)6 * (slab_planes(Lz, ctas) + 2) * Ly * Lh * elem + 15) / 16 * 16;
+}
+constexpr size_t kSlabBytes = 200 * 1024;  // slab and held sums together, of the 227 KB a CTA may have
 inline int held_passes(int precision, int threads) {
     const int fit = (int)(kHeldBytes / pass_bytes(precision, threads));
     return fit < 16 ? fit : 16;

@@ -16,7 +16,7 @@ from paper_2106_11286_gb300 import hs
 pytestmark = pytest.mark.gpu
 
 A6 = (0.1, -0.2, 0.05, 0.03, -0.04, 0.02)
-DIMS = [(2, 2, 2), (10, 6, 4), (12, 10, 14), (16, 16, 16), (18, 16, 18), (32, 16, 16), (48, 10, 50), (64, 32, 16),
+DIMS = [(2, 2, 2), (8, 4, 10), (20, 12, 18), (16, 32, 90), (10, 6, 4), (12, 10, 14), (16, 16, 16), (18, 16, 18), (32, 16, 16), (48, 10, 50), (64, 32, 16),
         (72, 64, 66)]
 LARGE = [(250, 62, 64), (128, 128, 182), (256, 184, 64)]
 
