@@ -628,16 +628,25 @@ __global__ void __launch_bounds__(kBlock) table_measure_kernel(const PassArgs a,
     for (int64_t i = t0; i < n_present; i += stride) {
         C h[3] = {C(0), C(0), C(0)}, hl[3] = {C(0), C(0), C(0)};
         const S4 sv = spins[i];
-#pragma unroll 4
-        for (int k = 0; k < a.width; ++k) {
-            const S4 n = spins[__ldg(a.nbr + (int64_t)k * a.n_pad + i)];
+        // four row entries, then their four gathers: two round trips per four neighbours (20 sweeps of a 3.1 M-site
+        // nanoparticle with this measurement 1136 -> 1115 us)
+        for (int k0 = 0; k0 < a.width; k0 += 4) {
+            S4 n[4];
+            int32_t j[4];
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                if constexpr (P == HS_FP64)
-                    h[q] += n.v[q];
-                else
-                    two_sum(h[q], hl[q], to_c(n.v[q]));
-            }
+            for (int k = 0; k < 4; ++k)
+                j[k] = k0 + k < a.width ? __ldg(a.nbr + (int64_t)(k0 + k) * a.n_pad + i) : (int32_t)n_present;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) n[k] = spins[j[k]];  // beyond the width: the zero dummy
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    if constexpr (P == HS_FP64)
+                        h[q] += n[k].v[q];
+                    else
+                        two_sum(h[q], hl[q], to_c(n[k].v[q]));
+                }
         }
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
