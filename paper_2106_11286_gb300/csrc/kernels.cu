@@ -361,12 +361,15 @@ __global__ void __launch_bounds__(kBlock, 2) sc_march_kernel(const PassArgs a) {
 // W > 0: a table of exactly W neighbours, unrolled: the W row entries load
 // together, then the W gathers, then the sums in stored order (the same
 // sums), so each site waits two round trips instead of 2 W.  It needs 64
-// registers (four CTAs per SM): at 48 the compiler issues the gathers one
-// after another again.  Measured on the FP32 bcc nanoparticle at W = 8:
-// 65.9 -> 76.9 attempts/ns without PFL2 (74.9 with it); a version that also
-// loaded the next site's row into registers measured lower.
+// registers (four CTAs per SM) at W = 8 in FP32: at 48 the compiler issues the
+// gathers one after another again.  Measured on the FP32 bcc nanoparticle at
+// W = 8: 65.9 -> 76.9 attempts/ns without PFL2 (74.9 with it); a version that
+// also loaded the next site's row into registers measured lower.  The trial is
+// drawn while the gathers travel: 144.7 -> 137.6 us per sweep there (76.3 ->
+// 80.2 attempts/ns), 44.8 -> 42.6 on one of 3.1 M sites; for the loop (W = 0),
+// whose gathers come one by one, after them (fcc FP32 37.9 against 44.0).
 template <int P, bool MEAS, bool TEN = false, bool PFL2 = false, int W = 0>
-__global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (W > 0 ? 4 : 5)) table_pass_kernel(const PassArgs a) {
+__global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (P == HS_FP32 && W == 8 ? 4 : 5)) table_pass_kernel(const PassArgs a) {
     pdl_enter();
     using S = typename Tr<P>::S;
     using C = typename Tr<P>::C;
@@ -378,6 +381,7 @@ __global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (W > 0 ? 4 : 5)) ta
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = a.begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.end; i += stride) {
         TableField<P, MEAS, TEN> f;
+        TableTrial<P> t;
         if (PFL2 && i + stride < a.end) {
             for (int k = 0; k < a.width; ++k)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(a.nbr + (int64_t)k * a.n_pad + i + stride));
@@ -390,6 +394,7 @@ __global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (W > 0 ? 4 : 5)) ta
             for (int k = 0; k < W; ++k) jj[k] = __ldg(a.nbr + (int64_t)k * a.n_pad + i);
 #pragma unroll
             for (int k = 0; k < W; ++k) nn[k] = spins[jj[k]];
+            draw_table_trial<P>(a, i, t);  // while the gathers are on their way
 #pragma unroll
             for (int k = 0; k < W; ++k) f.add(a, jj[k], nn[k]);
         } else {
@@ -399,8 +404,7 @@ __global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (W > 0 ? 4 : 5)) ta
             }
         }
         S4 s = spins[i];
-        TableTrial<P> t;
-        draw_table_trial<P>(a, i, t);
+        if constexpr (W == 0) draw_table_trial<P>(a, i, t);
         if (table_update<P, MEAS, TEN>(a, i, spins, f, t, s, J, K, ex, ey, ez, beta, acc)) spins[i] = s;
     }
     write_partials<C, MEAS>(a, acc.e, acc.x, acc.y, acc.z, acc.n);
@@ -954,6 +958,48 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t sme
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+cudaError_t launch_pdl_ptr(const void *kernel, int grid, int block, cudaStream_t s, const PassArgs &a) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    PassArgs args = a;
+    void *params[] = {&args};
+    return cudaLaunchKernelExC(&cfg, kernel, params);
+}
+
+// The neighbour-table kernel of a layout: unrolled rows for the crystals'
+// widths (FP32: 6 and 8; its 12 would hold 60 registers of neighbours; FP16,
+// whose spins are half as wide, 12 as well), a loop otherwise.  us per sweep,
+// loop and unrolled: FP16 fcc 70^3 42.5 and 33.9, bcc 90^3 27.9 and 23.3, open
+// sc 121^3 30.2 and 24.2; FP32 open sc 121^3 33.0 (with the L2 prefetch that it
+// had; 27.7 without) and 24.6.
+template <int P, int W, bool PFL2>
+const void *table_variant(bool meas) {
+    return meas ? (const void *)table_pass_kernel<P, true, false, PFL2, W>
+                : (const void *)table_pass_kernel<P, false, false, PFL2, W>;
+}
+template <int P>
+const void *table_kernel_ptr(const Layout &L, bool meas) {
+    if (L.tensor)
+        return meas ? (const void *)table_pass_kernel<P, true, true> : (const void *)table_pass_kernel<P, false, true>;
+    if constexpr (P == HS_FP32)
+        if (L.width == 8) return L.prefetch == 1 ? table_variant<P, 8, true>(meas) : table_variant<P, 8, false>(meas);
+    if (L.prefetch == 1) return table_variant<P, 0, true>(meas);
+    if constexpr (P != HS_FP64)
+        if (L.width == 6) return table_variant<P, 6, false>(meas);
+    if constexpr (P == HS_FP16) {
+        if (L.width == 8) return table_variant<P, 8, false>(meas);
+        if (L.width == 12) return table_variant<P, 12, false>(meas);
+    }
+    return table_variant<P, 0, false>(meas);
+}
+
 template <int P, int V, int PF>
 cudaError_t launch_sc_pf(const PassArgs &a, int n_blocks, cudaStream_t s, bool meas) {
     return meas ? launch_pdl(sc_pass_kernel<P, V, true, PF>, n_blocks, kBlock, 0, s, a)
@@ -1042,22 +1088,7 @@ cudaError_t launch_pass_p(const Layout &L, const PassArgs &a, int n_blocks, cuda
         }
         return cudaErrorInvalidValue;
     }
-    if (L.tensor)
-        return meas ? launch_pdl(table_pass_kernel<P, true, true>, n_blocks, kBlock, 0, s, a)
-                    : launch_pdl(table_pass_kernel<P, false, true>, n_blocks, kBlock, 0, s, a);
-    if constexpr (P == HS_FP32)
-        if (L.width == 8) {  // the unrolled 8-neighbour table (bcc, the nanoparticle's CSR)
-            if (L.prefetch == 1)
-                return meas ? launch_pdl(table_pass_kernel<P, true, false, true, 8>, n_blocks, kBlock, 0, s, a)
-                            : launch_pdl(table_pass_kernel<P, false, false, true, 8>, n_blocks, kBlock, 0, s, a);
-            return meas ? launch_pdl(table_pass_kernel<P, true, false, false, 8>, n_blocks, kBlock, 0, s, a)
-                        : launch_pdl(table_pass_kernel<P, false, false, false, 8>, n_blocks, kBlock, 0, s, a);
-        }
-    if (L.prefetch == 1)
-        return meas ? launch_pdl(table_pass_kernel<P, true, false, true>, n_blocks, kBlock, 0, s, a)
-                    : launch_pdl(table_pass_kernel<P, false, false, true>, n_blocks, kBlock, 0, s, a);
-    return meas ? launch_pdl(table_pass_kernel<P, true>, n_blocks, kBlock, 0, s, a)
-                : launch_pdl(table_pass_kernel<P, false>, n_blocks, kBlock, 0, s, a);
+    return launch_pdl_ptr(table_kernel_ptr<P>(L, meas), n_blocks, kBlock, s, a);
 }
 
 }  // namespace
@@ -1183,20 +1214,7 @@ static const void *pass_kernel_ptr(const Layout &L, bool meas) {
         }
         return nullptr;
     }
-    if (L.tensor)
-        return meas ? (const void *)table_pass_kernel<P, true, true> : (const void *)table_pass_kernel<P, false, true>;
-    if constexpr (P == HS_FP32)
-        if (L.width == 8) {
-            if (L.prefetch == 1)
-                return meas ? (const void *)table_pass_kernel<P, true, false, true, 8>
-                            : (const void *)table_pass_kernel<P, false, false, true, 8>;
-            return meas ? (const void *)table_pass_kernel<P, true, false, false, 8>
-                        : (const void *)table_pass_kernel<P, false, false, false, 8>;
-        }
-    if (L.prefetch == 1)
-        return meas ? (const void *)table_pass_kernel<P, true, false, true>
-                    : (const void *)table_pass_kernel<P, false, false, true>;
-    return meas ? (const void *)table_pass_kernel<P, true> : (const void *)table_pass_kernel<P, false>;
+    return table_kernel_ptr<P>(L, meas);
 }
 
 int pass_occupancy(int precision, const Layout &L, int accumulate) {
