@@ -175,11 +175,12 @@ GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, in
     const bool wide = precision == HS_FP64;
     if (!L.structured || L.slab || L.vec > 4 || L.n_sites > (wide ? kGridSites64 : kGridSites)) return none;
     const bool ten = L.tensor != 0, ax = zaxis != 0;
-    if (!ten && L.n_sites <= (wide ? kSlabSites64 : kSlabSites)) {
+    const int64_t items = L.n_sites / 2 / (wide ? 1 : L.vec);
+    if (!ten && items <= (wide ? kClusterItems64 : (L.vec == 1 ? kSlabItems1 : kSlabItems))) {
         const GroupPlan p = slab_plan(precision, L, ax, n_sm);
         if (p.ctas > 0) return p;
     }
-    if (L.n_sites <= (wide ? kClusterSites64 : kClusterSites)) {
+    if (items <= (wide ? kClusterItems64 : kClusterItems)) {
         GroupPlan p = none;
         if (wide) p.vec = 1;
         const int warps = (int)((L.n_sites / 2 / p.vec + 31) / 32);

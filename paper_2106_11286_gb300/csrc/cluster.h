@@ -5,20 +5,22 @@
 
 namespace hs {
 
-// The largest lattices that run in one cluster: beyond them its 16 SMs take
-// longer over a pass than a barrier over the whole device costs (us per sweep
-// FP32: 24^3 4.3 in the cluster, 32^3 5.1 there, 40^3 5.0 on the grid; FP64 16^3
-// 6.0 and 20^3 7.9 in the cluster, 24^3 7.2 on the grid).
-constexpr int64_t kClusterSites = 24000;   // FP32, FP16
-constexpr int64_t kClusterSites64 = 5000;  // FP64
+// The largest lattices that run in one cluster, by the work items of a pass:
+// beyond them its 16 SMs take longer than a barrier over the whole device
+// costs.  us per sweep in a cluster with the spins in its shared memory (slabs),
+// with them in L2, and on the grid:
+//   V = 4, FP32: 768 items 2.8, 4.3, 4.8; 4096 4.2, 5.1, 5.0; 6144 5.6, 6.0, 5.0
+//   V = 2, FP32: 3584 items 3.2, 3.9, 4.3; 9216 7.9, 9.6, 4.4
+//   V = 1, FP32: 1792 items 3.0, 3.8, 4.5; 2816 3.9, 3.9, 4.3; 3840 4.9, 4.4, 4.5
+//   FP64: 2048 items (16^3) 5.2, 6.0, 7; 4000 9.6, 7.9, 7.2
+constexpr int64_t kSlabItems = 4800;     // FP32, FP16
+constexpr int64_t kSlabItems1 = 3300;    // of one site each
+constexpr int64_t kClusterItems = 3600;
+constexpr int64_t kClusterItems64 = 2500;  // FP64, either way
 // The largest that run as one cooperative launch: beyond them the launches
 // are a small part of a pass (times in cluster.cu).
 constexpr int64_t kGridSites = 3000000;    // FP32, FP16
 constexpr int64_t kGridSites64 = 1000000;  // FP64
-
-// The largest that keep their spins in a cluster's shared memory.
-constexpr int64_t kSlabSites = 50000;   // FP32, FP16 (16^3 2.8 against 4.2, 32^3 4.2 against 5.1, 36^3 4.4 against 5.0)
-constexpr int64_t kSlabSites64 = 5000;  // FP64 (16^3 5.2 us per sweep against 6.0 with its spins in L2, 20^3 9.6 against 7.2 on the grid)
 
 // CTAs (0: the launch chain instead) of how many threads, sites per work item,
 // and how they run: one cluster with the spins in its shared memory or in L2,

@@ -4,7 +4,7 @@ spins bit for bit, the same accepted moves, and moments that differ by FP64
 rounding at most -- FP32 / FP16 sums are grouped alike, FP64 ones are added in
 another order, 10^4 terms of equal sign: below 1e-12.
 
-Sizes about the edges of the choice (24,000 and 5,000 sites, 3.0 and 1.0 million),
+Sizes about the edges of the choice (2500 to 4800 work items a pass, 3.0 and 1.0 million sites),
 of the warps and CTAs, of one or several items per thread, and of the vector
 widths; 70 sweeps, more than one group of 64, then one more call.
 """
@@ -16,7 +16,7 @@ from paper_2106_11286_gb300 import hs
 pytestmark = pytest.mark.gpu
 
 A6 = (0.1, -0.2, 0.05, 0.03, -0.04, 0.02)
-DIMS = [(2, 2, 2), (8, 4, 10), (20, 12, 18), (16, 32, 90), (10, 6, 4), (12, 10, 14), (16, 16, 16), (18, 16, 18), (32, 16, 16), (48, 10, 50), (64, 32, 16),
+DIMS = [(2, 2, 2), (8, 4, 10), (20, 12, 18), (16, 32, 90), (30, 16, 16), (36, 16, 64), (18, 20, 16), (40, 32, 24), (10, 6, 4), (12, 10, 14), (16, 16, 16), (18, 16, 18), (32, 16, 16), (48, 10, 50), (64, 32, 16),
         (72, 64, 66)]
 LARGE = [(250, 62, 64), (128, 128, 182), (256, 184, 64)]
 
