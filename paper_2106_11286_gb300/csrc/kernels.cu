@@ -368,8 +368,12 @@ __global__ void __launch_bounds__(kBlock, 2) sc_march_kernel(const PassArgs a) {
 // drawn while the gathers travel: 144.7 -> 137.6 us per sweep there (76.3 ->
 // 80.2 attempts/ns), 44.8 -> 42.6 on one of 3.1 M sites; for the loop (W = 0),
 // whose gathers come one by one, after them (fcc FP32 37.9 against 44.0).
-template <int P, bool MEAS, bool TEN = false, bool PFL2 = false, int W = 0>
-__global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (P == HS_FP32 && W == 8 ? 4 : 5)) table_pass_kernel(const PassArgs a) {
+// FP64 runs one CTA per SM (139 registers), or two (TWO: 128, with a few
+// spills) where a class has sites for them: fcc 864,000 sites 145.5 -> 117.3 us
+// per sweep, bcc 1,024,000 118.2 -> 92.7; fcc of 73,656 35.6 -> 50.4.
+template <int P, bool MEAS, bool TEN = false, bool PFL2 = false, int W = 0, bool TWO = false>
+__global__ void __launch_bounds__(kBlock, P == HS_FP64 ? (TWO ? 2 : 1) : (P == HS_FP32 && W == 8 ? 4 : 5))
+    table_pass_kernel(const PassArgs a) {
     pdl_enter();
     using S = typename Tr<P>::S;
     using C = typename Tr<P>::C;
@@ -979,10 +983,10 @@ cudaError_t launch_pdl_ptr(const void *kernel, int grid, int block, cudaStream_t
 // loop and unrolled: FP16 fcc 70^3 42.5 and 33.9, bcc 90^3 27.9 and 23.3, open
 // sc 121^3 30.2 and 24.2; FP32 open sc 121^3 33.0 (with the L2 prefetch that it
 // had; 27.7 without) and 24.6.
-template <int P, int W, bool PFL2>
+template <int P, int W, bool PFL2, bool TWO = false>
 const void *table_variant(bool meas) {
-    return meas ? (const void *)table_pass_kernel<P, true, false, PFL2, W>
-                : (const void *)table_pass_kernel<P, false, false, PFL2, W>;
+    return meas ? (const void *)table_pass_kernel<P, true, false, PFL2, W, TWO>
+                : (const void *)table_pass_kernel<P, false, false, PFL2, W, TWO>;
 }
 template <int P>
 const void *table_kernel_ptr(const Layout &L, bool meas) {
@@ -996,6 +1000,11 @@ const void *table_kernel_ptr(const Layout &L, bool meas) {
     if constexpr (P == HS_FP16) {
         if (L.width == 8) return table_variant<P, 8, false>(meas);
         if (L.width == 12) return table_variant<P, 12, false>(meas);
+    }
+    if constexpr (P == HS_FP64) {
+        int64_t most = 0;  // sites of the largest class
+        for (int c = 0; c < L.n_colours; ++c) most = std::max(most, L.colour_begin[c + 1] - L.colour_begin[c]);
+        if (most > 152 * kBlock) return table_variant<P, 0, false, true>(meas);
     }
     return table_variant<P, 0, false>(meas);
 }

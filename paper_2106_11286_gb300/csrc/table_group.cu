@@ -23,7 +23,7 @@ namespace hs {
 namespace {
 
 template <int P, bool MEAS, int W>
-__global__ void __launch_bounds__(kBlock, P == HS_FP64 ? 1 : (W > 8 ? 2 : 3)) table_group_kernel(const PassArgs args,
+__global__ void __launch_bounds__(kBlock, P == HS_FP64 || W > 8 ? 2 : 3) table_group_kernel(const PassArgs args,
                                                                                    const TableClasses cls, int n_sweeps,
                                                                                    int depth,
                                                                                    unsigned long long arrivals) {
