@@ -252,7 +252,7 @@ def run_ours(args):
     mom, count = lat.read_accumulator()
     # Mean launch duration of the dominant kernel from the CUDA events of the
     # timed region: it holds colour-pass launches of that kernel (2 per step)
-    # and the ring folds of the fused sums (two small launches per fold_sweeps
+    # and the ring folds of the fused sums (one small launch per fold_sweeps
     # steps), so region time / launches, inter-launch gaps included, bounds the
     # achieved bandwidth from below.  A second, identical run with
     # every launch bracketed by its own events is reported beside it (those
@@ -346,8 +346,8 @@ def run_ours(args):
     if rank != 0:
         return None
     # kernels launched in one timed region: two colour passes per sweep and the ring folds of the fused
-    # sums (a per-sweep sum kernel and an apply kernel per fold_sweeps sweeps)
-    gpu_launches = 2 * args.steps + 2 * ((args.steps + fold - 1) // fold)
+    # sums (one kernel per fold_sweeps sweeps)
+    gpu_launches = 2 * args.steps + (args.steps + fold - 1) // fold
     cpu, spin_err = (None, None) if (args.no_cpu_baseline or world > 1) else cpu_baseline(args)
     precision = None if (args.no_precision or world > 1) else precision_runs(args)
     tc = None if (args.no_precision or world > 1) else tc_runs(args)

@@ -245,7 +245,11 @@ int hs_read_timing(hs_lattice *h, double *ms, int64_t *launches);
 /* Launch configuration of the colour-pass kernels (the autotuner's knobs).
  * Results never depend on it: a site's random numbers and arithmetic are
  * fixed by its natural index, so every configuration gives bit-identical
- * spins.  Zero fields mean "choose automatically". */
+ * spins.  Zero fields mean "choose automatically".  With every field zero,
+ * hs_sweep runs a small lattice (sc up to 3 million sites, 1 million in FP64;
+ * neighbour tables of 6, 8 or 12 neighbours up to 600,000 sites, without the
+ * tensor term) as one launch per group of sweeps, with the named kernel's
+ * arithmetic and sums, unless hs_enable_timing counts its passes' launches. */
 enum hs_kernel {
     HS_KERNEL_AUTO = 0,
     HS_KERNEL_STENCIL = 1, /* sc: operands loaded through L1/L2 into registers */
@@ -272,7 +276,7 @@ typedef struct {
                           0 = automatic (off);
                           table: 1 = ask L2 for the next site's table row
                           and spin ahead, 2 = off, 0 = automatic (on for FP32
-                          tables of fewer than 8 neighbours) */
+                          tables of fewer than 8 neighbours, but not 6) */
     int order;         /* stencil: order of the work items over a sweep:
                           1 = every pass in ascending (z, y, x) order,
                           2 = alternating (the passes of colour 1 descending,
@@ -358,7 +362,9 @@ void hs_batch_destroy(hs_batch *b);
  * memory once and stay there for every sweep, the colour passes separated
  * by CTA barriers only (no grid barrier, no global traffic between the
  * first load and the final store; the work split and load schedule do not
- * apply), for n_trial_sweeps sweeps at the given
+ * apply) -- or, for FP64 batches of at most half as many members as SMs, of
+ * at most 16384 sites each, one cluster of several CTAs per member -- for
+ * n_trial_sweeps sweeps at the given
  * betas after one warm-up sweep; the fastest is kept.  Colour 0 then colour
  * 1 in every sweep under all of them.  Every member's spins, sweep counter
  * and accumulator are restored, so the members' chains are as if the call
@@ -367,7 +373,7 @@ void hs_batch_destroy(hs_batch *b);
  * hs_batch_get_layout reads the choice in use (hs_batch_create starts with
  * the maximum CTAs per SM, the interleaved split (align_rows 2), no
  * prefetch, and schedule 2 when there are at least 16 members and every one
- * fits in a CTA's shared memory, else schedule 0). */
+ * fits in a CTA's shared memory, or each gets a cluster, else schedule 0). */
 int hs_batch_autotune(hs_batch *b, const double *betas, int n_trial_sweeps);
 int hs_batch_get_layout(const hs_batch *b, int *ctas_per_sm, int *align_rows, int *prefetch, int *schedule);
 /* Set the choice by hand: ctas_per_sm in 1 .. the kernel's occupancy,

@@ -231,7 +231,7 @@ __device__ __forceinline__ void batch_pass(const BatchArgs &b, int s, int c) {
             for (uint32_t t = sg.begin + threadIdx.x; t < sg.end; t += sg.stride) {
                 StencilItem<P, V> it;
                 load_item<P, V, CG>(a, t, own, oth, it);
-                if (update_item<P, V, true, false, AX, CG>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p,
+                if (update_item<P, V, true, false, AX, CG, P == HS_FP32>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p,
                                                            it.site0, it.rank0, c, a, J, K, ex, ey, ez, beta, acc, oth,
                                                            it.b0)) {
 #pragma unroll
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(kBlock, 2) batch_resident_kernel(const BatchAr
             for (uint32_t t = threadIdx.x; t < n_items; t += kBlock) {
                 StencilItem<P, V> it;
                 load_item<P, V>(a, t, own, oth, it);
-                if (update_item<P, V, true, false, AX>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0,
+                if (update_item<P, V, true, false, AX, false, P != HS_FP64>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0,
                                                        it.rank0, c, a, J, K, ex, ey, ez, beta, acc, oth, it.b0)) {
 #pragma unroll
                     for (int q = 0; q < 3; ++q) *reinterpret_cast<VT *>(own_w[q] + it.b0) = it.s[q];

@@ -119,32 +119,39 @@ void group_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int p
     cfg.numAttrs = 2;
 }
 
-// The device takes kernel k as p asks.
-bool ask_fits(int precision, const GroupPlan &p, const void *k, int n_sm) {
+// How many of p's clusters, or of its CTAs per SM, the device holds at once.
+int ask_held(int precision, const GroupPlan &p, const void *k) {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[2];
     group_config(cfg, attr, precision, p, nullptr);
     int n = 0;
-    bool ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(p.kind == kGroupSlabs ? kSlabBytes : kHeldBytes)) == cudaSuccess;
-    if (ok && p.kind == kGroupGrid) {
-        ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, p.threads, cfg.dynamicSmemBytes) == cudaSuccess &&
-             n * n_sm >= p.ctas;
-    } else if (ok) {
+    cudaError_t e;
+    if (p.kind == kGroupGrid) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, p.threads, cfg.dynamicSmemBytes);
+    } else {
         cfg.numAttrs = 1;
-        ok = (p.ctas <= 8 || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
-             cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n >= 1;
+        e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
     }
-    if (!ok) cudaGetLastError();
-    return ok;
+    if (e == cudaSuccess) return n;
+    cudaGetLastError();
+    return 0;
 }
 
 // Both variants (with and without the fused measurement) fit the device as p asks.
 bool plan_fits(int precision, const GroupPlan &p, bool ten, bool ax, int n_sm) {
     for (int meas = 0; meas < 2; ++meas) {
         const void *k = group_kernel(precision, p, meas != 0, ten, ax);
-        if (!k || cached_fit(k, p.ctas, p.threads + (int)(p.smem / 1024) * 1024, [&] { return ask_fits(precision, p, k, n_sm) ? 1 : 0; }) == 0)
+        if (!k) return false;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(p.kind == kGroupSlabs ? kSlabBytes : kHeldBytes)) != cudaSuccess ||
+            (p.kind != kGroupGrid && p.ctas > 8 &&
+             cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+            cudaGetLastError();
             return false;
+        }
+        const int n = cached_fit(k, p.kind == kGroupGrid ? 0 : p.ctas, p.threads + (int)(p.smem / 1024) * 1024,
+                                 [&] { return ask_held(precision, p, k); });
+        if (p.kind == kGroupGrid ? n * n_sm < p.ctas : n < 1) return false;
     }
     return true;
 }

@@ -1,7 +1,7 @@
-// What the driver answers about a kernel and a launch shape on a device, kept
-// for the life of the process: the questions (function attributes, occupancy)
-// cost a lattice's creation some 80 us, a fifth of it, and their answers
-// depend on nothing else.  One entry per variant and shape; any thread.
+// What the driver answers about a kernel's occupancy at a launch shape on a
+// device, kept for the life of the process: the questions cost a lattice's
+// creation some 80 us, a fifth of it, and their answers depend on nothing else.
+// One entry per variant and shape; any thread.
 #pragma once
 
 #include <cuda_runtime.h>

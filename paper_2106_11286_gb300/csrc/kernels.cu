@@ -71,14 +71,16 @@ __global__ void __launch_bounds__(kBlock, 2) sc_pass_kernel(const PassArgs a) {
     const S *const oth[3] = {(const S *)a.oth[0], (const S *)a.oth[1], (const S *)a.oth[2]};
     SiteAcc<P> acc;
     const uint32_t stride = gridDim.x * blockDim.x;
+    // slabs offset the ranks by whole planes, which hold a multiple of V sites: pairs stay pairs
+    constexpr bool kEarly = P == HS_FP16 && V <= 4 && PF == 0 && DIR;
     auto compute = [&](StencilItem<P, V> &it) {
         bool any;
         if constexpr (P == HS_FP64)
             any = update_item<P, V, MEAS, TEN, AX>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0,
                                                    it.rank0, c, a, J, K, ex, ey, ez, beta, acc, oth, it.b0);
         else
-            any = update_item<P, V, MEAS, TEN, AX>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p, it.site0,
-                                                   it.rank0, c, a, J, K, ex, ey, ez, beta, acc);
+            any = update_item<P, V, MEAS, TEN, AX, false, kEarly>(it.s, it.o, it.nym, it.nyp, it.nzm, it.nzp, it.ed, it.p,
+                                                                  it.site0, it.rank0, c, a, J, K, ex, ey, ez, beta, acc);
         if (any) {
 #pragma unroll
             for (int q = 0; q < 3; ++q) *reinterpret_cast<VT *>(own_w[q] + it.b0) = it.s[q];

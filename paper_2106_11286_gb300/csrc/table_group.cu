@@ -142,15 +142,19 @@ TableGroupPlan table_group_plan(int precision, const Layout &L, int n_blocks, in
         const void *k = table_group(precision, L.width, meas != 0);
         auto ask = [&] {
             int n = 0;
-            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeldBytes) != cudaSuccess ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, p.threads, table_held_bytes(precision, p.threads)) !=
-                    cudaSuccess) {
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, p.threads, table_held_bytes(precision, p.threads)) !=
+                cudaSuccess) {
                 cudaGetLastError();
                 return 0;
             }
             return n;
         };
-        if (!k || cached_fit(k, 0, p.threads, ask) * n_sm < ctas) return p;
+        if (!k) return p;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeldBytes) != cudaSuccess) {
+            cudaGetLastError();
+            return p;
+        }
+        if (cached_fit(k, 0, p.threads, ask) * n_sm < ctas) return p;
     }
     p.ctas = ctas;
     return p;
