@@ -58,8 +58,15 @@
  *     natural site order, 3 values per site (x, y, z), for all n_sites
  *     natural indices; absent (masked) sites read back as 0 and are ignored
  *     on input.
- *   - A device-side error (a bounded wait that timed out) is latched on the
- *     device and reported by the next call that synchronises.
+ *   - A device-side error (a bounded wait that timed out: between the colour
+ *     passes of hs_sweep's group launches, hs_set_launch, or of
+ *     hs_batch_run) is latched on the device and reported once, as
+ *     HS_E_TIMEOUT, by the next hs_measure, hs_read_accumulator or
+ *     hs_read_sums; the spin read-backs do not report it.  What the same
+ *     hs_sweep call has queued behind the wait that ran out leaves at once:
+ *     the spins stay as they were then, part-way through a sweep, no further
+ *     sweep is added to the accumulator, and the sweep counter has advanced
+ *     by the whole call.  The context and the handle stay usable.
  */
 #ifndef HS_H
 #define HS_H
@@ -535,13 +542,18 @@ int hs_read_sums(hs_lattice *h, double out[5]);
  * frees a small device buffer; synchronous.  HS_E_INVALID for another kind. */
 int hs_measure_alu_peak(int kind, void *cuda_stream, double *flops_per_s);
 
-/* Test hook for the bounded device-side waits (failure detection without a
- * GPU fault): in the next hs_batch_run (persistent schedule) one CTA skips
+/* Test hooks for the bounded device-side waits (failure detection without a
+ * GPU fault).  hs_inject_timeout: the next hs_sweep of the handle that runs a
+ * group of sweeps behind a grid barrier (hs_set_launch) waits at its first
+ * barrier for one arrival too many, so every CTA's bounded wait runs out
+ * together (about one second); see "A device-side error" above for what
+ * follows.  hs_batch_inject_timeout: in the next hs_batch_run (persistent schedule) one CTA skips
  * its first grid-barrier arrival, so every other CTA's bounded wait runs out
  * (about one second).  The kernel latches its error word and returns; the
  * next synchronising call on each member reports HS_E_TIMEOUT and clears it,
  * the CUDA context stays usable, and the spins of the interrupted sweep are
  * left part-updated. */
+int hs_inject_timeout(hs_lattice *h, int on);
 int hs_batch_inject_timeout(hs_batch *b, int on);
 
 const char *hs_last_error(void);

@@ -208,6 +208,7 @@ struct hs_lattice {
     Layout L{};
     int n_blocks = 1;
     hs_launch req{};        // requested launch configuration (0 = automatic)
+    int inject_timeout = 0;  // test hook, consumed by the next hs_sweep whose launches wait on a grid barrier
     hs::GroupPlan group{0, 0, 1, hs::kGroupCluster, 0, 0};  // small lattices' automatic launch: a whole group of sweeps at once
     int max_blocks = 1;     // capacity of the partials buffer
     int fold_ring = 1;      // sweeps per ring fold (slot sets of the partials buffer)
@@ -454,6 +455,7 @@ int configure_launch(hs_lattice *h) {
             const hs::TableGroupPlan p = hs::table_group_plan(h->precision, L, h->n_blocks, h->n_sm);
             h->group.ctas = p.ctas;
             h->group.threads = p.threads;
+            h->group.kind = hs::kGroupGrid;
         }
         return HS_OK;
     }
@@ -840,6 +842,10 @@ int hs_sweep(hs_lattice *h, double beta, int64_t n_sweeps) {
     if (h->group.ctas > 0 && !h->timing) {  // (timing counts the colour passes' own launches)
         a.n_blocks = h->group.ctas;
         unsigned long long arrivals = 0;
+        if (h->inject_timeout && h->group.kind == hs::kGroupGrid) {
+            arrivals = 1;  // test hook: one arrival that nobody makes
+            h->inject_timeout = 0;
+        }
         for (int64_t s = 0; s < n_sweeps;) {
             const int k = (int)std::min<int64_t>(h->fold_ring, n_sweeps - s);
             a.sweep = (uint32_t)(h->sweep + (uint64_t)s);
@@ -2007,6 +2013,12 @@ int hs_batch_get_layout(const hs_batch *b, int *ctas_per_sm, int *align_rows, in
 }
 
 void hs_batch_destroy(hs_batch *b) { delete b; }
+
+int hs_inject_timeout(hs_lattice *h, int on) {
+    if (!h) return fail(HS_E_INVALID, "null handle");
+    h->inject_timeout = on ? 1 : 0;
+    return HS_OK;
+}
 
 int hs_batch_inject_timeout(hs_batch *b, int on) {
     if (!b) return fail(HS_E_INVALID, "null handle");

@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) sc_slab_kernel(const PassA
 template <int P, int V, bool MEAS, int AX, bool TEN>
 __global__ void __launch_bounds__(kBlock, 2) sc_grid_kernel(const PassArgs args, void *planes, int n_sweeps,
                                                             int alternate, int depth, unsigned long long arrivals) {
+    if (abandoned(&args.acc->passed)) return;
     sweep_group<P, V, MEAS, AX, TEN, true>(args, planes, n_sweeps, alternate, depth, arrivals, (int)blockIdx.x,
                                              (int)gridDim.x);
 }

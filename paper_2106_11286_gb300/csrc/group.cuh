@@ -74,7 +74,10 @@ constexpr long long kBarrierCycles = 2000000000LL;  // about one second
 // The barrier between two passes.  Cluster: the hardware's.  Grid: a count of
 // arrivals in device memory that only grows (zeroed by hs_sweep); thread 0
 // arrives for its CTA with a release, and polls with acquires for at most
-// about a second, after which it latches the error word and every CTA leaves.
+// about a second, after which it latches the error word and marks the count
+// abandoned.  The mark ends the waits of the other CTAs, and the launches that
+// the same call has queued behind this one, whose targets the count can no
+// longer reach, leave as they start (abandoned) with their folds (kernels.cu).
 template <bool GRID>
 struct PassBarrier {
     unsigned long long *count;
@@ -99,10 +102,15 @@ struct PassBarrier {
                 const long long t0 = clock64();
                 for (uint32_t it = 0;; ++it) {
                     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
+                    if (v & kAbandoned) {
+                        ok = 0;
+                        break;
+                    }
                     if (v >= target) break;
                     if (it > (1u << 30) || clock64() - t0 > kBarrierCycles) {
                         ok = 0;
                         atomicExch(error, 1);
+                        atomicOr(count, kAbandoned);
                         break;
                     }
                 }
@@ -116,6 +124,12 @@ struct PassBarrier {
         }
     }
 };
+
+// A wait of this hs_sweep call ran out: in an earlier launch, or in another CTA
+// of this one before this CTA started.  The same answer for the whole CTA.
+__device__ __forceinline__ bool abandoned(const unsigned long long *count) {
+    return __syncthreads_or(threadIdx.x == 0 && (*(volatile const unsigned long long *)count & kAbandoned) != 0) != 0;
+}
 
 // n_sweeps sweeps of one lattice by its ctas CTAs (the whole grid, or one
 // cluster), of which this is number cta.  Work item t of a pass belongs to

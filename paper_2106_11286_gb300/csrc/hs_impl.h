@@ -52,12 +52,14 @@ struct FastDiv {
 #endif
 };
 
+constexpr unsigned long long kAbandoned = 1ull << 63;  // in DevAccum::passed: a wait of this hs_sweep call ran out
+
 // Device-resident accumulator block of one lattice.
 struct DevAccum {
     double moments[HS_N_MOMENTS];
     double count;          // accumulated sweeps
     double accepted;       // accepted moves since the last hs_sweep began
-    unsigned long long passed;  // CTA arrivals at the pass barrier of a cooperative sweep launch since then
+    unsigned long long passed;  // CTA arrivals at the pass barrier of a cooperative sweep launch since then (kAbandoned)
     double last[8];        // E, Mx, My, Mz, |M|, M2, M4, |M.e| of the last finalised reduction
     unsigned int done;     // CTA arrival counter of the finishing pass
     int error;             // latched device error code (0 = none)

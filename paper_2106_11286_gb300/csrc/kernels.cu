@@ -740,6 +740,8 @@ __device__ void fold_apply(const PassArgs &a, int n_slots) {
 __global__ void __launch_bounds__(kBlock) fold_kernel(const PassArgs a) {
     __shared__ int s_last;
     pdl_enter();
+    // the group launch before it gave up (kAbandoned): its slots are incomplete, and nothing of them is added
+    if (__ldcg(&a.acc->passed) & kAbandoned) return;
     double tot[kPartials];
     slot_totals<kBlock>(a, blockIdx.x, tot);
     if (threadIdx.x == 0) {

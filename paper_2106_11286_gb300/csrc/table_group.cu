@@ -31,6 +31,7 @@ __global__ void __launch_bounds__(kBlock, P == HS_FP64 || W > 8 ? 2 : 3) table_g
     using C = typename Tr<P>::C;
     using S4 = Vec<S, 4>;
     extern __shared__ __align__(16) unsigned char table_smem[];
+    if (abandoned(&args.acc->passed)) return;
     PassArgs a = args;
     PassSums held;
     held.warps = (int)blockDim.x / 32;
