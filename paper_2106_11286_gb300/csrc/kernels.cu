@@ -419,54 +419,70 @@ __global__ void __launch_bounds__(kBlock, P == HS_FP64 ? (TWO ? 2 : 1) : (P == H
 // ----------------------------------------------------------------- measure
 // Standalone Eq. 1 / Eq. 2 of the current state to FP64 accuracy.
 //
-// FP32 / FP16 storage works in unevaluated pairs of floats: every addition
+// FP32 / FP16 storage sums in unevaluated triples of floats: every addition
 // keeps its rounding error (TwoSum, Knuth, The Art of Computer Programming
-// vol. 2, 4.2.2) and every product its remainder (one fma), so a site's share
-// carries 48 bits and a thread's sums lose nothing that FP64 sums of the same
-// numbers would keep; the FP64 pipe, which issues 2 instructions per cycle
-// per SM against 128 for FP32, is left with one conversion per thread.  The
-// plain FP64 form, 45 FP64 instructions and 21 conversions a site, took
-// 2059 us at 256^3 and 12177 us at 464^3 FP32; a whole case of ten 464^3
-// sweeps, a measurement and the spins' read-back went from 19.08 to 7.35 ms
-// with this one (FP16 19.30 to 7.80, the 3.1 M-site nanoparticle 1.50 to 1.17).
+// vol. 2, 4.2.2), whose own sum keeps its errors in turn, and every product its
+// remainder (one fma), so a thread's sums carry 72 bits where FP64's carry 53;
+// a field of six neighbours is a pair, exact for components of 2^-20 and more
+// (or 0), off by 2^-45 at most where one is smaller.  The FP64 pipe, which
+// issues 2 instructions per cycle per SM against 128 for FP32, is left with
+// the threads' totals.  A whole hs_measure, us: 256^3 FP32 140, FP16 155; 464^3
+// 621 and 747.  With FP64 throughout, 45 FP64 instructions and 21 conversions a
+// site, 2102 and 12224; in pairs of floats, too few bits, 116 and 498 (FP32).
 // On the sc stencil every bond is counted once, at its colour-1 site, from the
 // vector loads of the sweep's work items; colour 0 adds its own spins only.
 template <typename T>
 __device__ __forceinline__ T sub_exact(T a, T b) { return f_fma(splat<T>(-1.0f), b, a); }  // a - b, one rounding
 
-// a + v with the rounding error added to lo
+// a += v; returns the rounding error
 template <typename T>
-__device__ __forceinline__ void two_sum(T &a, T &lo, T v) {
+__device__ __forceinline__ T two_sum(T &a, T v) {
     const T s = f_add(a, v);
     const T bb = sub_exact(s, a);
     const T e = f_add(sub_exact(a, sub_exact(s, bb)), sub_exact(v, bb));
     a = s;
-    lo = f_add(lo, e);
+    return e;
 }
 
-// sum += s (hh + hl), the product's remainder kept in lo
+// A sum a + b + c: b holds what a's additions left over, c what b's did.
 template <typename T>
-__device__ __forceinline__ void two_prod_add(T &sum, T &lo, T s, T hh, T hl) {
-    const T p = f_mul(s, hh);
-    const T r = f_fma(s, hh, f_mul(splat<T>(-1.0f), p));
-    lo = f_add(lo, f_fma(s, hl, r));
-    two_sum(sum, lo, p);
-}
-
-// Sums of one thread: bonds, (S.e)^2 and the spin components, as pairs.
-template <typename T>
-struct PairSums {
-    T b, bl, k, kl, m[3], ml[3];
-    __device__ __forceinline__ PairSums() {
-        b = bl = k = kl = splat<T>(0.0f);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) m[q] = ml[q] = splat<T>(0.0f);
+struct Sum3 {
+    T a = splat<T>(0.0f), b = splat<T>(0.0f), c = splat<T>(0.0f);
+    __device__ __forceinline__ void add_rest(T v) { c = f_add(c, two_sum(b, v)); }
+    __device__ __forceinline__ void add(T v) { add_rest(two_sum(a, v)); }
+    __device__ __forceinline__ void add_square(T s) {
+        const T p = f_mul(s, s);
+        add(p);
+        add_rest(f_fma(s, s, f_mul(splat<T>(-1.0f), p)));
     }
+    // s (hh + hl)
+    __device__ __forceinline__ void add_product(T s, T hh, T hl) {
+        const T p = f_mul(s, hh), q = f_mul(s, hl);
+        add(p);
+        add_rest(f_fma(s, hh, f_mul(splat<T>(-1.0f), p)));
+        add_rest(q);
+        c = f_add(c, f_fma(s, hl, f_mul(splat<T>(-1.0f), q)));
+    }
+    __device__ __forceinline__ double value() const;
 };
-__device__ __forceinline__ double wide_sum(float h, float l) { return (double)h + (double)l; }
-__device__ __forceinline__ double wide_sum(float2 h, float2 l) {
-    return wide_sum(h.x, l.x) + wide_sum(h.y, l.y);
+template <>
+__device__ __forceinline__ double Sum3<float>::value() const { return (double)a + ((double)b + (double)c); }
+template <>
+__device__ __forceinline__ double Sum3<float2>::value() const {
+    return ((double)a.x + (double)a.y) + (((double)b.x + (double)b.y) + ((double)c.x + (double)c.y));
 }
+
+// Sums of one thread: bonds, (S.e)^2 and the spin components.
+template <typename T>
+struct TripleSums {
+    Sum3<T> b, k, m[3];
+};
+
+// FP32's products hold their remainders down to 2^-126: a thread's sum below this is taken again in FP64.
+constexpr double kSmallSum = 0x1p-70;
+
+__device__ __forceinline__ uint32_t bits_of(float v) { return __float_as_uint(v); }
+__device__ __forceinline__ uint32_t bits_of(float2 v) { return __float_as_uint(v.x) | __float_as_uint(v.y); }
 
 template <typename T, typename S, int V>
 __device__ __forceinline__ T lanes(const Vec<S, V> &v, int j) {
@@ -541,15 +557,17 @@ __global__ void __launch_bounds__(kBlock) sc_measure_kernel(const PassArgs a, co
     } else {
         using T = typename std::conditional<(V >= 2), float2, float>::type;
         constexpr int W = V >= 2 ? V / 2 : 1;  // lane groups of an item
-        PairSums<T> A;
+        TripleSums<T> A;
+        uint32_t zbits = 0;  // of every S_z: none but zeros leave k at 0 exactly
         auto own = [&](const VT (&s)[3]) {
 #pragma unroll
             for (int j = 0; j < W; ++j) {
 #pragma unroll
-                for (int q = 0; q < 3; ++q) two_sum(A.m[q], A.ml[q], lanes<T>(s[q], j));
+                for (int q = 0; q < 3; ++q) A.m[q].add(lanes<T>(s[q], j));
                 if (!GEN) {
                     const T z = lanes<T>(s[2], j);
-                    two_prod_add(A.k, A.kl, z, z, splat<T>(0.0f));
+                    A.k.add_square(z);
+                    zbits |= bits_of(z);
                 }
             }
             if (GEN)
@@ -579,22 +597,23 @@ __global__ void __launch_bounds__(kBlock) sc_measure_kernel(const PassArgs a, co
                     } else {
                         x = it.ed[q];
                     }
-                    T h = lanes<T>(it.o[q], j), hl = splat<T>(0.0f);
-                    two_sum(h, hl, x);
-                    two_sum(h, hl, lanes<T>(it.nym[q], j));
-                    two_sum(h, hl, lanes<T>(it.nyp[q], j));
-                    two_sum(h, hl, lanes<T>(it.nzm[q], j));
-                    two_sum(h, hl, lanes<T>(it.nzp[q], j));
-                    two_prod_add(A.b, A.bl, lanes<T>(it.s[q], j), h, hl);
+                    T h = lanes<T>(it.o[q], j), hl;
+                    hl = two_sum(h, x);
+                    hl = f_add(hl, two_sum(h, lanes<T>(it.nym[q], j)));
+                    hl = f_add(hl, two_sum(h, lanes<T>(it.nyp[q], j)));
+                    hl = f_add(hl, two_sum(h, lanes<T>(it.nzm[q], j)));
+                    hl = f_add(hl, two_sum(h, lanes<T>(it.nzp[q], j)));
+                    A.b.add_product(lanes<T>(it.s[q], j), h, hl);
                 }
             own(it.s);
         }
-        double b = wide_sum(A.b, A.bl), k = wide_sum(A.k, A.kl);
+        double b = A.b.value(), k = A.k.value();
         double m[3];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) m[q] = wide_sum(A.m[q], A.ml[q]);
-        // beyond FP32's range (no unit vectors): the same sums in FP64
-        if (!(isfinite(b) && isfinite(k) && isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]))) {
+        for (int q = 0; q < 3; ++q) m[q] = A.m[q].value();
+        // beyond FP32's range, or so small that it held no remainders (no unit vectors): the same sums in FP64
+        const bool small = P == HS_FP32 && (fabs(b) < kSmallSum || (!GEN && k < kSmallSum && (zbits << 1) != 0u));
+        if (small || !(isfinite(b) && isfinite(k) && isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]))) {
             b = k = m[0] = m[1] = m[2] = accG = 0.0;
             for (uint64_t t = t0; t < n_items; t += stride) {
                 StencilItem<P, V> it;
@@ -634,7 +653,7 @@ __global__ void __launch_bounds__(kBlock) table_measure_kernel(const PassArgs a,
     double b = 0, g = 0, m[3] = {0, 0, 0};
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    PairSums<float> A;
+    TripleSums<float> A;
     for (int64_t i = t0; i < n_present; i += stride) {
         C h[3] = {C(0), C(0), C(0)}, hl[3] = {C(0), C(0), C(0)};
         const S4 sv = spins[i];
@@ -655,7 +674,7 @@ __global__ void __launch_bounds__(kBlock) table_measure_kernel(const PassArgs a,
                     if constexpr (P == HS_FP64)
                         h[q] += n[k].v[q];
                     else
-                        two_sum(h[q], hl[q], to_c(n[k].v[q]));
+                        hl[q] = f_add(hl[q], two_sum(h[q], to_c(n[k].v[q])));
                 }
         }
 #pragma unroll
@@ -665,17 +684,18 @@ __global__ void __launch_bounds__(kBlock) table_measure_kernel(const PassArgs a,
                 b = fma(s, h[q], b);
                 m[q] += s;
             } else {
-                two_prod_add(A.b, A.bl, s, h[q], hl[q]);
-                two_sum(A.m[q], A.ml[q], s);
+                A.b.add_product(s, h[q], hl[q]);
+                A.m[q].add(s);
             }
         }
         if (onsite) g += onsite64(a, to_c(sv.v[0]), to_c(sv.v[1]), to_c(sv.v[2]));
     }
     if constexpr (P != HS_FP64) {
-        b = wide_sum(A.b, A.bl);
+        b = A.b.value();
 #pragma unroll
-        for (int q = 0; q < 3; ++q) m[q] = wide_sum(A.m[q], A.ml[q]);
-        if (!(isfinite(b) && isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]))) {  // beyond FP32's range
+        for (int q = 0; q < 3; ++q) m[q] = A.m[q].value();
+        const bool small = P == HS_FP32 && fabs(b) < kSmallSum;
+        if (small || !(isfinite(b) && isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]))) {  // as above
             b = m[0] = m[1] = m[2] = 0.0;
             for (int64_t i = t0; i < n_present; i += stride)
                 for (int q = 0; q < 3; ++q) {
