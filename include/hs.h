@@ -542,6 +542,13 @@ int hs_read_sums(hs_lattice *h, double out[5]);
  * frees a small device buffer; synchronous.  HS_E_INVALID for another kind. */
 int hs_measure_alu_peak(int kind, void *cuda_stream, double *flops_per_s);
 
+/* FP64 lattices take a move's decision from an FP32 value of beta dH wherever
+ * that value is farther from the threshold -ln P than its error bound, which
+ * this returns for sites of n_neighbours neighbours (J, K, beta as given), and
+ * from FP64 elsewhere: the decisions are FP64's.  Infinite where J, K or beta
+ * leave FP32's range: FP64 decides every site.  Host only. */
+double hs_decision_band(double beta, double J, double K, int n_neighbours);
+
 /* Test hooks for the bounded device-side waits (failure detection without a
  * GPU fault).  hs_inject_timeout: the next hs_sweep of the handle that runs a
  * group of sweeps behind a grid barrier (hs_set_launch) waits at its first

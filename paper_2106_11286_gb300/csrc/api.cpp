@@ -2014,6 +2014,10 @@ int hs_batch_get_layout(const hs_batch *b, int *ctas_per_sm, int *align_rows, in
 
 void hs_batch_destroy(hs_batch *b) { delete b; }
 
+double hs_decision_band(double beta, double J, double K, int n_neighbours) {
+    return (double)hs::decision_band(beta, J, K, n_neighbours);
+}
+
 int hs_inject_timeout(hs_lattice *h, int on) {
     if (!h) return fail(HS_E_INVALID, "null handle");
     h->inject_timeout = on ? 1 : 0;

@@ -148,22 +148,25 @@ struct Layout {
 
 // How far the FP32 form of beta dH may be from the FP64 one, for spins whose
 // components are at most 1 + 2^-12 (of any length: unit vectors stay well
-// inside) and six neighbours at most.  In units of 2^-24, per field component:
-// six operands truncated to FP32 (2 each) and five additions of sums up to 6 (6
-// each), 42; so S.h is off by at most 3 42 + 2 18 (S truncated) + 3 18 (the
-// products' roundings) = 216, S'.h by less, and J (S.h - S'.h) by 2 216 + 36 +
-// 2 36 = 540 < 4e-5 / 2^-24 = 671; a field taken from FP64 is closer.  Up to
-// twelve neighbours (the table's fcc): fields up to 12, eleven additions, 156
-// per component, 1512 in all < 1.2e-4 / 2^-24 = 2013.  The uniaxial term: S.e
-// off by 12 each, times a sum of at most 3.5, with its roundings below 200 <
-// 2e-5 / 2^-24 = 335.  Infinite (FP64 decides every site) where J, K or beta
-// leave FP32's range.
+// inside) and w neighbours.  In units of 2^-24, per field component: w operands
+// truncated to FP32 (2 each) and w - 1 additions of sums up to w (w each),
+// w^2 + w at most; so S.h is off by at most 3 (w^2 + w) + 6 w (S truncated) +
+// 9 w (the products' roundings), S'.h by less, and J (S.h - S'.h) by twice that
+// + 6 w + 12 w: 6 w^2 + 54 w in all (540 for six neighbours, 3.2e-5; 1512 for
+// fcc's twelve), a quarter more for what exceeds 1; a field taken from FP64 is
+// closer.  The uniaxial term: S.e off by 12 each, times a sum of at most 3.5,
+// with its roundings below 200 < 2e-5 / 2^-24 = 335.  Infinite (FP64 decides
+// every site) where J, K or beta leave FP32's range.  No width is left out: a
+// table of 14 neighbours whose sites FP64 all decided took its gathers twice,
+// 103 us per sweep of 27,648 sites against 90 without the FP32 form, and 54 with
+// it deciding (26 neighbours 211, 169 and 101; 1,024,000 sites of 14 259, 258
+// and 127).
 inline float decision_band(double beta, double J, double K, int width) {
     auto fits = [](double v) { return v == 0.0 || (v >= 1e-30 && v <= 1e30); };
     const double aJ = J < 0 ? -J : J, aK = K < 0 ? -K : K;
-    if (!fits(beta) || !fits(aJ) || !fits(aK) || !fits(beta * aJ) || !fits(beta * aK) || width > 12)
-        return __builtin_inff();
-    return (float)(beta * (aJ * (width > 6 ? 1.2e-4 : 4e-5) + aK * 2e-5) * 1.001);
+    if (!fits(beta) || !fits(aJ) || !fits(aK) || !fits(beta * aJ) || !fits(beta * aK)) return __builtin_inff();
+    const double w = width, units = 1.25 * (6.0 * w * w + 54.0 * w);
+    return (float)(beta * (aJ * units * 0x1p-24 + aK * 2e-5) * 1.001);
 }
 
 // Fewer items than the SMs have threads of one CTA each: CTAs of as few warps

@@ -113,6 +113,7 @@ SIGNATURES = {
     "hs_sweep_sc_fp32_noalloc": (ctypes.c_int, [_vp, _i32p, ctypes.POINTER(hs_params), ctypes.c_double,
                                                  ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint64, ctypes.c_int64,
                                                  _vp, _vp]),
+    "hs_decision_band": (ctypes.c_double, [ctypes.c_double, ctypes.c_double, ctypes.c_double, ctypes.c_int]),
     "hs_inject_timeout": (ctypes.c_int, [_vp, ctypes.c_int]),
     "hs_batch_inject_timeout": (ctypes.c_int, [_vp, ctypes.c_int]),
     "hs_measure_alu_peak": (ctypes.c_int, [ctypes.c_int, _vp, ctypes.POINTER(ctypes.c_double)]),
@@ -502,6 +503,10 @@ def hs_batch_set_layout(b, ctas_per_sm, align_rows=0, prefetch=0, schedule=0):
 
 def hs_batch_destroy(b):
     load().hs_batch_destroy(b)
+
+
+def hs_decision_band(beta, J, K, n_neighbours) -> float:
+    return float(load().hs_decision_band(float(beta), float(J), float(K), int(n_neighbours)))
 
 
 def hs_inject_timeout(h, on=True):
