@@ -298,6 +298,19 @@ typedef struct {
 int hs_set_launch(hs_lattice *h, const hs_launch *cfg);
 int hs_get_launch(const hs_lattice *h, hs_launch *out);
 
+/* How hs_sweep launches a group of sweeps at once under the configuration in
+ * force (hs_get_launch names the colour passes' kernel and CTAs): not at all
+ * (kind HS_GROUP_NONE, the rest 0), in one thread-block cluster with the spins
+ * in L2 or in its CTAs' shared memory, or in one cooperative launch. */
+enum hs_group_kind { HS_GROUP_NONE = 0, HS_GROUP_CLUSTER = 1, HS_GROUP_SLABS = 2, HS_GROUP_GRID = 3 };
+typedef struct {
+    int kind;    /* hs_group_kind */
+    int ctas;
+    int threads; /* of a CTA */
+    int vec;     /* sites per work item */
+} hs_group_launch;
+int hs_get_group_launch(const hs_lattice *h, hs_group_launch *out);
+
 /* On-site anisotropy tensor: adds -sum_i S_i^T A S_i to Eq. 1 (to dH in
  * Metropolis step (iii), to E in hs_measure and in the fused per-sweep
  * reductions), with A symmetric, given as its six entries

@@ -1307,12 +1307,14 @@ int hs_set_launch(hs_lattice *h, const hs_launch *cfg) {
     const hs_launch keep = h->req;
     const Layout keep_l = h->L;
     const int keep_b = h->n_blocks;
+    const hs::GroupPlan keep_g = h->group;
     h->req = *cfg;
     int st = configure_launch(h);
     if (st) {
         h->req = keep;
         h->L = keep_l;
         h->n_blocks = keep_b;
+        h->group = keep_g;
     }
     return st;
 }
@@ -1333,6 +1335,7 @@ int hs_set_anisotropy_tensor(hs_lattice *h, const double A[6]) {
     const hs_launch keep_req = h->req;
     const Layout keep_l = h->L;
     const int keep_b = h->n_blocks;
+    const hs::GroupPlan keep_g = h->group;
     h->tensor = on;
     for (int q = 0; q < 6; ++q) h->tA[q] = t[q];
     h->req = hs_launch{};  // back to the automatic launch, which takes the tensor into account
@@ -1343,6 +1346,7 @@ int hs_set_anisotropy_tensor(hs_lattice *h, const double A[6]) {
         h->req = keep_req;
         h->L = keep_l;
         h->n_blocks = keep_b;
+        h->group = keep_g;
     }
     return st;
 }
@@ -1364,6 +1368,18 @@ int hs_get_launch(const hs_lattice *h, hs_launch *out) {
                         ? (L.prefetch == 1 ? 1 : (L.prefetch == 2 ? 3 : 2))
                         : 0;
     out->order = L.kernel == hs::kStencil ? L.order : 0;
+    return HS_OK;
+}
+
+int hs_get_group_launch(const hs_lattice *h, hs_group_launch *out) {
+    if (!h || !out) return fail(HS_E_INVALID, "null argument");
+    const hs::GroupPlan &g = h->group;
+    *out = hs_group_launch{HS_GROUP_NONE, 0, 0, 0};
+    if (g.ctas > 0)
+        *out = hs_group_launch{g.kind == hs::kGroupGrid    ? HS_GROUP_GRID
+                               : g.kind == hs::kGroupSlabs ? HS_GROUP_SLABS
+                                                           : HS_GROUP_CLUSTER,
+                               g.ctas, g.threads, h->L.structured ? g.vec : 1};
     return HS_OK;
 }
 

@@ -52,6 +52,12 @@ class hs_launch(ctypes.Structure):
         return {k: getattr(self, k) for k, _ in self._fields_}
 
 
+class hs_group_launch(ctypes.Structure):
+    _fields_ = [("kind", ctypes.c_int), ("ctas", ctypes.c_int), ("threads", ctypes.c_int), ("vec", ctypes.c_int)]
+
+
+GROUP_KINDS = {0: "none", 1: "cluster", 2: "slabs", 3: "grid"}
+
 HS_KERNEL_AUTO, HS_KERNEL_STENCIL, HS_KERNEL_TABLE, HS_KERNEL_MARCH, HS_KERNEL_PIPE = 0, 1, 3, 4, 5
 KERNELS = {"auto": 0, "stencil": 1, "table": 3, "march": 4, "pipe": 5}
 
@@ -99,6 +105,7 @@ SIGNATURES = {
     "hs_read_timing": (ctypes.c_int, [_vp, _dp, _i64p]),
     "hs_set_launch": (ctypes.c_int, [_vp, ctypes.POINTER(hs_launch)]),
     "hs_get_launch": (ctypes.c_int, [_vp, ctypes.POINTER(hs_launch)]),
+    "hs_get_group_launch": (ctypes.c_int, [_vp, ctypes.POINTER(hs_group_launch)]),
     "hs_set_anisotropy_tensor": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_double)]),
     "hs_get_anisotropy_tensor": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_double)]),
     "hs_autotune": (ctypes.c_int, [_vp, ctypes.c_double, ctypes.c_int]),
@@ -391,6 +398,12 @@ def hs_get_launch(h) -> dict:
     return cfg.as_dict()
 
 
+def hs_get_group_launch(h) -> dict:
+    g = hs_group_launch()
+    _check(load().hs_get_group_launch(h, ctypes.byref(g)))
+    return {"kind": GROUP_KINDS[g.kind], "ctas": g.ctas, "threads": g.threads, "vec": g.vec}
+
+
 def tensor_entries(A):
     """The six entries (Axx, Ayy, Azz, Axy, Axz, Ayz) of a symmetric on-site
     anisotropy tensor given as six numbers or a symmetric 3x3 array."""
@@ -593,6 +606,10 @@ class Lattice:
     @property
     def launch(self):
         return hs_get_launch(self.h)
+
+    @property
+    def group_launch(self):
+        return hs_get_group_launch(self.h)
 
     @property
     def info(self):

@@ -1,0 +1,26 @@
+"""Which launch runs a small lattice's sweeps (hs_get_group_launch), and that
+the configuration calls leave it as it was where they say that they change
+nothing."""
+import pytest
+
+from paper_2106_11286_gb300 import hs
+
+pytestmark = pytest.mark.gpu
+
+SMALL = [("sc", (16, 16, 16), "fp64"), ("sc", (24, 24, 24), "fp32"), ("sc", (18, 20, 16), "fp16"),
+         ("sc", (64, 64, 64), "fp32"), ("sc", (32, 32, 32), "fp64"), ("bcc", (20, 20, 20), "fp32"),
+         ("fcc", (12, 12, 12), "fp64")]
+
+
+@pytest.mark.parametrize("kind,dims,precision", SMALL)
+def test_a_refused_configuration_changes_nothing(kind, dims, precision):
+    with hs.Lattice(kind, dims=dims, precision=precision) as lat:
+        launch, group = lat.launch, lat.group_launch
+        assert group["kind"] != "none" and group["ctas"] > 0
+        refused = [dict(prefetch=3)] if kind != "sc" else [dict(kernel="march", tile_y=7), dict(kernel="table")]
+        if precision == "fp16" and kind == "sc":
+            refused.append(dict(kernel="pipe", vec_width=1))  # 2 bytes a vector
+        for bad in refused:
+            with pytest.raises(hs.HSError):
+                lat.set_launch(**bad)
+            assert (lat.launch, lat.group_launch) == (launch, group)
