@@ -294,7 +294,9 @@ typedef struct {
 } hs_launch;
 
 /* Set (fields 0 = automatic) or read the launch configuration.  Kernel
- * codes 2 and 6 are not used (HS_E_INVALID). */
+ * codes 2 and 6 are not used (HS_E_INVALID).  What hs_get_launch returns of an
+ * automatic configuration names it whole: setting it again restores the
+ * automatic choice, the group launch with it. */
 int hs_set_launch(hs_lattice *h, const hs_launch *cfg);
 int hs_get_launch(const hs_lattice *h, hs_launch *out);
 

@@ -1285,6 +1285,13 @@ int hs_read_timing(hs_lattice *h, double *ms, int64_t *launches) {
 }
 
 // ---------------------------------------------------------------- launch configuration
+namespace {
+bool same_launch(const hs_launch &a, const hs_launch &b) {
+    return std::tie(a.kernel, a.vec_width, a.blocks_per_sm, a.tile_y, a.prefetch, a.order) ==
+           std::tie(b.kernel, b.vec_width, b.blocks_per_sm, b.tile_y, b.prefetch, b.order);
+}
+}  // namespace
+
 int hs_set_launch(hs_lattice *h, const hs_launch *cfg) {
     if (!h || !cfg) return fail(HS_E_INVALID, "null argument");
     if (cfg->kernel != HS_KERNEL_AUTO && cfg->kernel != HS_KERNEL_STENCIL && cfg->kernel != HS_KERNEL_TABLE &&
@@ -1308,6 +1315,13 @@ int hs_set_launch(hs_lattice *h, const hs_launch *cfg) {
     const Layout keep_l = h->L;
     const int keep_b = h->n_blocks;
     const hs::GroupPlan keep_g = h->group;
+    // the automatic choice under its full name, as hs_get_launch gives it, is the automatic choice
+    if (cfg->kernel != HS_KERNEL_AUTO && !h->L.slab) {
+        hs_launch automatic;
+        h->req = hs_launch{};
+        if (configure_launch(h) == HS_OK && hs_get_launch(h, &automatic) == HS_OK && same_launch(automatic, *cfg))
+            return HS_OK;
+    }
     h->req = *cfg;
     int st = configure_launch(h);
     if (st) {

@@ -24,3 +24,19 @@ def test_a_refused_configuration_changes_nothing(kind, dims, precision):
             with pytest.raises(hs.HSError):
                 lat.set_launch(**bad)
             assert (lat.launch, lat.group_launch) == (launch, group)
+
+
+@pytest.mark.parametrize("kind,dims,precision", SMALL + [("sc", (200, 200, 200), "fp32"), ("sc", (20, 16, 6), "fp64")])
+def test_a_saved_configuration_restores_the_launch(kind, dims, precision):
+    with hs.Lattice(kind, dims=dims, precision=precision) as lat:
+        launch, group = lat.launch, lat.group_launch
+        lat.set_launch(**launch)
+        assert (lat.launch, lat.group_launch) == (launch, group)
+        lat.set_launch(**dict(kernel="stencil", order=1) if kind == "sc" else dict(kernel="table", blocks_per_sm=1))
+        assert lat.group_launch["kind"] == "none"
+        lat.set_launch(**launch)
+        assert (lat.launch, lat.group_launch) == (launch, group)
+        lat.set_launch(kernel="stencil" if kind == "sc" else "table")
+        assert lat.group_launch["kind"] == "none"  # a kernel named: its launch chain
+        lat.set_launch()
+        assert (lat.launch, lat.group_launch) == (launch, group)
