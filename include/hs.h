@@ -256,7 +256,10 @@ int hs_read_timing(hs_lattice *h, double *ms, int64_t *launches);
  * hs_sweep runs a small lattice (sc up to 3 million sites, 1 million in FP64;
  * neighbour tables of 6, 8 or 12 neighbours up to 600,000 sites, without the
  * tensor term) as one launch per group of sweeps, with the named kernel's
- * arithmetic and sums, unless hs_enable_timing counts its passes' launches. */
+ * arithmetic and sums, unless hs_enable_timing counts its passes' launches.  On
+ * a stream of its own (not the default stream) a lattice takes that launch only
+ * where the device holds four like it, so that lattices on several streams
+ * sweep side by side. */
 enum hs_kernel {
     HS_KERNEL_AUTO = 0,
     HS_KERNEL_STENCIL = 1, /* sc: operands loaded through L1/L2 into registers */

@@ -432,6 +432,20 @@ int clear_slab_sets(hs_lattice *h) {
     return HS_OK;
 }
 
+// How many cooperative launches like a lattice's the device must hold at once
+// for its sweeps to run that way.  Lattices on the default stream run one after
+// another: one.  A lattice on a stream of its own may have others sweeping
+// beside it, whose passes fill each other's latencies as launch chains do and
+// as grids that hold every SM through their barriers cannot: four.  us per
+// lattice and sweep, group and chain, of 1, 2, 4, 8 lattices on streams of
+// their own: FP32 48^3 (five fit) 6.2 and 9.3, 3.4 and 4.9, 2.1 and 2.8, 1.8 and
+// 2.2; 64^3 (two) 6.2 and 9.0, 3.8 and 4.9, 3.5 and 3.3, 3.4 and 3.1; 96^3 (one)
+// 10.6 and 12.5, 10.3 and 7.7, 10.2 and 7.5, 10.2 and 8.0; bcc 28^3 (five) 5.0
+// and 7.3 ... 1.6 and 2.1; bcc 40^3 (one) 5.5 and 9.7, 5.4 and 5.2, 5.2 and 3.0,
+// 5.2 and 2.8; FP64 32^3 (four) 8.2 and 18.1, 4.8 and 11.6, 3.9 and 6.2, 3.9 and 3.6;
+// 64^3 (one) 21.8 and 27.0, 21.1 and 17.6, 20.9 and 16.4, 20.7 and 16.5.
+int group_room(const hs_lattice *h) { return h->stream == nullptr || h->stream == cudaStreamLegacy ? 1 : 4; }
+
 int configure_launch(hs_lattice *h) {
     Layout &L = h->L;
     if (L.slab && (h->sets_written != 0 || h->interior_due >= 0))
@@ -452,7 +466,7 @@ int configure_launch(hs_lattice *h) {
         if (bps <= 0 || bps > occ) bps = occ;
         h->n_blocks = std::min(hs::pass_blocks(h->precision, L, h->n_sm, bps), h->max_blocks);
         if (r.kernel == HS_KERNEL_AUTO && r.blocks_per_sm == 0 && r.prefetch == 0) {
-            const hs::TableGroupPlan p = hs::table_group_plan(h->precision, L, h->n_blocks, h->n_sm);
+            const hs::TableGroupPlan p = hs::table_group_plan(h->precision, L, h->n_blocks, h->n_sm, group_room(h));
             h->group.ctas = p.ctas;
             h->group.threads = p.threads;
             h->group.kind = hs::kGroupGrid;
@@ -522,7 +536,7 @@ int configure_launch(hs_lattice *h) {
     if (bps <= 0 || bps > occ) bps = occ;
     h->n_blocks = std::min(hs::pass_blocks(h->precision, L, h->n_sm, bps), h->max_blocks);
     if (r.kernel == HS_KERNEL_AUTO && r.vec_width == 0 && r.blocks_per_sm == 0 && r.prefetch == 0 && r.order == 0)
-        h->group = hs::group_plan(h->precision, L, z_axis(h), h->n_blocks, h->n_sm);
+        h->group = hs::group_plan(h->precision, L, z_axis(h), h->n_blocks, h->n_sm, group_room(h));
     return clear_slab_sets(h);  // the parts' grids follow the launch configuration
 }
 

@@ -139,7 +139,7 @@ int ask_held(int precision, const GroupPlan &p, const void *k) {
 }
 
 // Both variants (with and without the fused measurement) fit the device as p asks.
-bool plan_fits(int precision, const GroupPlan &p, bool ten, bool ax, int n_sm) {
+bool plan_fits(int precision, const GroupPlan &p, bool ten, bool ax, int n_sm, int room) {
     for (int meas = 0; meas < 2; ++meas) {
         const void *k = group_kernel(precision, p, meas != 0, ten, ax);
         if (!k) return false;
@@ -152,7 +152,7 @@ bool plan_fits(int precision, const GroupPlan &p, bool ten, bool ax, int n_sm) {
         }
         const int n = cached_fit(k, p.kind == kGroupGrid ? 0 : p.ctas, p.threads + (int)(p.smem / 1024) * 1024,
                                  [&] { return ask_held(precision, p, k); });
-        if (p.kind == kGroupGrid ? n * n_sm < p.ctas : n < 1) return false;
+        if (p.kind == kGroupGrid ? n * n_sm < p.ctas * room : n < 1) return false;
     }
     return true;
 }
@@ -172,13 +172,13 @@ GroupPlan slab_plan(int precision, const Layout &L, bool ax, int n_sm) {
         if (p.smem + pass_bytes(precision, p.threads) > kSlabBytes) continue;
         p.depth = (int)std::min<size_t>(held_passes(precision, p.threads),
                                         (kSlabBytes - p.smem) / pass_bytes(precision, p.threads));
-        if (plan_fits(precision, p, false, ax, n_sm)) return p;
+        if (plan_fits(precision, p, false, ax, n_sm, 1)) return p;
     }
     return GroupPlan{0, 0, L.vec, kGroupCluster, 0, 0};
 }
 }  // namespace
 
-GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, int n_sm) {
+GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, int n_sm, int room) {
     const GroupPlan none{0, 0, L.vec, kGroupCluster, 0, 0};
     const bool wide = precision == HS_FP64;
     if (!L.structured || L.slab || L.vec > 4 || L.n_sites > (wide ? kGridSites64 : kGridSites)) return none;
@@ -197,7 +197,7 @@ GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, in
             if (p.ctas > warps && p.ctas > 1) continue;
             p.threads = std::min(kClusterThreads, 32 * ((warps + p.ctas - 1) / p.ctas));
             p.depth = held_passes(precision, p.threads);
-            if (plan_fits(precision, p, ten, ax, n_sm)) return p;
+            if (plan_fits(precision, p, ten, ax, n_sm, 1)) return p;
         }
         return none;
     }
@@ -208,7 +208,7 @@ GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, in
     }
     spread_ctas(L.n_sites / 2 / p.vec, n_sm, p.ctas, p.threads);
     p.depth = held_passes(precision, p.threads);
-    return plan_fits(precision, p, ten, ax, n_sm) ? p : none;
+    return plan_fits(precision, p, ten, ax, n_sm, room) ? p : none;
 }
 
 cudaError_t launch_group(int precision, const Layout &L, const GroupPlan &p, const PassArgs &a, int n_sweeps,

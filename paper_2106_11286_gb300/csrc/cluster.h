@@ -32,7 +32,8 @@ struct GroupPlan {
     size_t smem;
     int depth;
 };
-GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, int n_sm);
+// room: how many such cooperative launches the device must hold at once (group_room).
+GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, int n_sm, int room);
 
 // n_sweeps sweeps from a.sweep on, sweep s to ring slot s; a.n_blocks = p.ctas,
 // arrivals: those already counted in a.acc->passed.

@@ -132,7 +132,7 @@ size_t table_held_bytes(int precision, int threads) {
 
 }  // namespace
 
-TableGroupPlan table_group_plan(int precision, const Layout &L, int n_blocks, int n_sm) {
+TableGroupPlan table_group_plan(int precision, const Layout &L, int n_blocks, int n_sm, int room) {
     TableGroupPlan p{0, kBlock};
     if (L.structured || L.tensor || L.n_present < 1 || L.n_present > kTableGroupSites) return p;
     int64_t items = 0;
@@ -155,7 +155,7 @@ TableGroupPlan table_group_plan(int precision, const Layout &L, int n_blocks, in
             cudaGetLastError();
             return p;
         }
-        if (cached_fit(k, 0, p.threads, ask) * n_sm < ctas) return p;
+        if (cached_fit(k, 0, p.threads, ask) * n_sm < ctas * room) return p;
     }
     p.ctas = ctas;
     return p;

@@ -15,11 +15,12 @@ struct TableClasses {
 
 // CTAs of the launch and their threads (the launch chain's n_blocks of kBlock,
 // or spread_ctas), ctas 0 where it does not apply: the tensor term, widths
-// other than 6, 8 and 12, larger lattices, or a grid not resident at once.
+// other than 6, 8 and 12, larger lattices, or fewer than room such grids
+// resident at once (group_room).
 struct TableGroupPlan {
     int ctas, threads;
 };
-TableGroupPlan table_group_plan(int precision, const Layout &L, int n_blocks, int n_sm);
+TableGroupPlan table_group_plan(int precision, const Layout &L, int n_blocks, int n_sm, int room);
 cudaError_t launch_table_group(int precision, const Layout &L, const PassArgs &a, const TableGroupPlan &p,
                                int n_sweeps, unsigned long long arrivals, cudaStream_t s);
 

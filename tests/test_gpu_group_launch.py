@@ -2,6 +2,7 @@
 the configuration calls leave it as it was where they say that they change
 nothing."""
 import pytest
+import torch
 
 from paper_2106_11286_gb300 import hs
 
@@ -40,3 +41,21 @@ def test_a_saved_configuration_restores_the_launch(kind, dims, precision):
         assert lat.group_launch["kind"] == "none"  # a kernel named: its launch chain
         lat.set_launch()
         assert (lat.launch, lat.group_launch) == (launch, group)
+
+
+@pytest.mark.parametrize("kind,dims,precision,own", [
+    ("sc", (16, 16, 16), "fp64", "slabs"), ("sc", (24, 24, 24), "fp32", "cluster"), ("sc", (48, 48, 48), "fp32", "grid"),
+    ("sc", (24, 24, 24), "fp64", "grid"), ("bcc", (20, 20, 20), "fp32", "grid"), ("fcc", (12, 12, 12), "fp64", "grid"),
+    ("sc", (64, 64, 64), "fp32", "none"), ("sc", (96, 96, 96), "fp32", "none"), ("sc", (96, 96, 96), "fp16", "none"),
+    ("sc", (64, 64, 64), "fp64", "none"), ("bcc", (40, 40, 40), "fp32", "none"), ("fcc", (36, 36, 36), "fp32", "none")])
+def test_a_stream_of_its_own_leaves_room(kind, dims, precision, own):
+    """Four cooperative launches fit the device at once, or the sweeps stay a chain; the default stream's lattices,
+    which run one after another, take what one fits."""
+    with hs.Lattice(kind, dims=dims, precision=precision) as lat, \
+            hs.Lattice(kind, dims=dims, precision=precision, stream=torch.cuda.Stream()) as beside:
+        assert beside.group_launch["kind"] == own
+        assert lat.group_launch["kind"] == (own if own != "none" else "grid")
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        if own == "grid":  # 128 registers a thread at most, 65536 an SM
+            g = beside.group_launch
+            assert 4 * g["ctas"] <= sms * (2048 // g["threads"])
