@@ -253,13 +253,15 @@ int hs_read_timing(hs_lattice *h, double *ms, int64_t *launches);
  * Results never depend on it: a site's random numbers and arithmetic are
  * fixed by its natural index, so every configuration gives bit-identical
  * spins.  Zero fields mean "choose automatically".  With every field zero,
- * hs_sweep runs a small lattice (sc up to 3 million sites, 1 million in FP64;
- * neighbour tables of 6, 8 or 12 neighbours up to 600,000 sites, without the
- * tensor term) as one launch per group of sweeps, with the named kernel's
- * arithmetic and sums, unless hs_enable_timing counts its passes' launches.  On
- * a stream of its own (not the default stream) a lattice takes that launch only
- * where the device holds four like it, so that lattices on several streams
- * sweep side by side. */
+ * hs_sweep runs a small lattice (sc: in FP32 up to 3 million sites, 300,000
+ * where Lx/2 is odd; in FP16 2.5 million, 920,000 where Lx/2 is not a multiple
+ * of 4 and 300,000 where it is odd; in FP64 1 million; neighbour tables of 6, 8
+ * or 12 neighbours up to 600,000 sites, in FP32 and FP16 as far as the device
+ * holds a thread for every site of a class, without the tensor term) as one
+ * launch per group of sweeps, with the named kernel's arithmetic and sums,
+ * unless hs_enable_timing counts its passes' launches.  On a stream of its own
+ * (not the default stream) a lattice takes that launch only where the device
+ * holds four like it, so that lattices on several streams sweep side by side. */
 enum hs_kernel {
     HS_KERNEL_AUTO = 0,
     HS_KERNEL_STENCIL = 1, /* sc: operands loaded through L1/L2 into registers */

@@ -67,7 +67,11 @@ cudaError_t launch_batch_resident(int precision, const BatchArgs &b, size_t smem
 size_t batch_resident_limit(int precision);
 // the resident schedule of FP64 batches of few members: one cluster of ctas
 // CTAs (0: none) of that many threads per member, for members of at most
-// kBatchClusterSites sites (24^3 measured 2.5 times the persistent schedule)
+// kBatchClusterSites sites: us per sweep in clusters and on the persistent
+// schedule, of 12, 24, 48 and 76 members of 24^3 (13,824 sites) 20.2 and 30.6, 27.1
+// and 35.5, 52.5 and 55.5, 52.4 and 69.7; of 16,384 sites 20.5 and 28.8, 32.3 and
+// 39.1, 63.0 and 58.5, 58.7 and 71.9; of 24,576 27.0 and 31.0, 39.8 and 45.9, 77.7 and
+// 72.3, 83.6 and 94.6; of 32^3 32.7 and 40.9, 51.4 and 57.6, 101 and 84, 109 and 117
 constexpr int64_t kBatchClusterSites = 16384;
 struct BatchClusters {
     int ctas, threads;

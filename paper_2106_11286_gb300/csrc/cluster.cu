@@ -18,12 +18,12 @@
 // the launch chain: 16^3 FP64 6.0 and 15.6, 16^3 FP32 4.2 and 6.7, 24^3 FP32 4.3
 // and 6.8.
 //
-// Lattices of up to kGridSites sites run the same loop on the whole device as
+// Lattices of up to some million sites (cluster.h) run the same loop on the whole device as
 // one cooperative launch, with a barrier over the grid: it takes about as long
 // as the cluster's plus one atomic and one poll, still less than ending a
 // launch and starting the next: 64^3 FP32 5.4 and 8.6 us per sweep, 96^3 10.0
-// and 11.9, 128^3 15.9 and 18.3, 160^3 27.4 and 27.6; FP64 32^3 7.2 and 16.7,
-// 64^3 20.5 and 26.2, 96^3 46.2 and 48.4, 128^3 94.0 and 92.3.
+// and 11.9, 128^3 15.9 and 18.3; FP64 32^3 7.2 and 16.7, 64^3 20.5 and 26.2, 96^3
+// 46.2 and 48.4.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -178,10 +178,20 @@ GroupPlan slab_plan(int precision, const Layout &L, bool ax, int n_sm) {
 }
 }  // namespace
 
+namespace {
+// Sites up to which a lattice of this precision and width sweeps in groups (cluster.h has the times on both sides).
+int64_t group_sites(int precision, int vec) {
+    if (precision == HS_FP64) return kGridSites64;
+    if (vec == 1) return 2 * kGridItems1;
+    if (precision == HS_FP32) return kGridSites;
+    return vec == 2 ? 4 * kGridItems2 : kGridSites16;
+}
+}  // namespace
+
 GroupPlan group_plan(int precision, const Layout &L, int zaxis, int n_blocks, int n_sm, int room) {
     const GroupPlan none{0, 0, L.vec, kGroupCluster, 0, 0};
     const bool wide = precision == HS_FP64;
-    if (!L.structured || L.slab || L.vec > 4 || L.n_sites > (wide ? kGridSites64 : kGridSites)) return none;
+    if (!L.structured || L.slab || L.vec > 4 || L.n_sites > group_sites(precision, L.vec)) return none;
     const bool ten = L.tensor != 0, ax = zaxis != 0;
     const int64_t items = L.n_sites / 2 / (wide ? 1 : L.vec);
     if (!ten && items <= (wide ? kClusterItems64 : (L.vec == 1 ? kSlabItems1 : kSlabItems))) {

@@ -1,6 +1,7 @@
 """Which launch runs a small lattice's sweeps (hs_get_group_launch), and that
 the configuration calls leave it as it was where they say that they change
 nothing."""
+import numpy as np
 import pytest
 import torch
 
@@ -59,3 +60,48 @@ def test_a_stream_of_its_own_leaves_room(kind, dims, precision, own):
         if own == "grid":  # 128 registers a thread at most, 65536 an SM
             g = beside.group_launch
             assert 4 * g["ctas"] <= sms * (2048 // g["threads"])
+
+
+@pytest.mark.parametrize("kind,dims,precision,group", [
+    # work items about the clusters' lines: 4096 and 4608 of four sites, 2816 and 3840 of one
+    ("sc", (32, 32, 32), "fp32", "slabs"), ("sc", (32, 32, 36), "fp32", "grid"), ("sc", (32, 32, 32), "fp16", "slabs"),
+    ("sc", (32, 32, 36), "fp16", "grid"), ("sc", (22, 16, 16), "fp32", "slabs"), ("sc", (30, 16, 16), "fp32", "grid"),
+    ("sc", (28, 28, 18), "fp32", "cluster"), ("sc", (28, 28, 24), "fp32", "grid"),
+    ("sc", (16, 16, 18), "fp64", "slabs"), ("sc", (20, 16, 16), "fp64", "grid"), ("sc", (20, 16, 6), "fp64", "cluster"),
+    # about the cooperative launch's: by width in FP32 and FP16
+    ("sc", (144, 144, 144), "fp32", "grid"), ("sc", (152, 144, 144), "fp32", "none"),
+    ("sc", (124, 116, 116), "fp32", "grid"), ("sc", (70, 54, 70), "fp32", "grid"), ("sc", (70, 70, 72), "fp32", "none"),
+    ("sc", (136, 136, 128), "fp16", "grid"), ("sc", (136, 136, 144), "fp16", "none"),
+    ("sc", (92, 92, 90), "fp16", "grid"), ("sc", (100, 100, 98), "fp16", "none"),
+    ("sc", (70, 54, 70), "fp16", "grid"), ("sc", (70, 70, 72), "fp16", "none"),
+    ("sc", (96, 96, 96), "fp64", "grid"), ("sc", (100, 102, 100), "fp64", "none"),
+    # neighbour tables: what is resident at once in FP32 and FP16, the stated number of sites in FP64
+    ("bcc", (48, 48, 48), "fp32", "grid"), ("bcc", (50, 50, 50), "fp32", "none"), ("bcc", (48, 48, 48), "fp16", "grid"),
+    ("bcc", (50, 50, 50), "fp16", "none"), ("fcc", (42, 42, 42), "fp32", "grid"), ("fcc", (43, 43, 43), "fp32", "none"),
+    ("bcc", (66, 66, 66), "fp64", "grid"), ("bcc", (67, 67, 67), "fp64", "none")])
+def test_the_launch_by_size(kind, dims, precision, group):
+    """Each kind of launch on both sides of its lines, so that the comparisons with the chain compare what they say."""
+    with hs.Lattice(kind, dims=dims, precision=precision) as lat:
+        assert lat.group_launch["kind"] == group, lat.group_launch
+
+
+@pytest.mark.parametrize("kind,dims,precision", [
+    ("sc", (70, 54, 70), "fp32"), ("sc", (70, 54, 70), "fp16"), ("sc", (92, 92, 90), "fp16"),  # several items a thread
+    ("bcc", (48, 48, 48), "fp32"), ("bcc", (48, 48, 48), "fp16"), ("fcc", (42, 42, 42), "fp32"),  # every SM full
+    ("bcc", (66, 66, 66), "fp64")])
+def test_the_largest_groups_equal_the_chain(kind, dims, precision):
+    """As in test_gpu_group.py: spins and accepted moves bit for bit, moments within the FP64 rounding of their sums."""
+    got = []
+    for chain in (False, True):
+        with hs.Lattice(kind, dims=dims, precision=precision, seed=8, K=0.2, e=(0.3, -0.2, 1.0)) as lat:
+            if chain:
+                lat.set_launch(kernel="stencil" if kind == "sc" else "table")
+            assert (lat.group_launch["kind"] == "none") == chain
+            lat.init()
+            lat.accumulate(True)
+            lat.sweep(0.8, 3)
+            got.append((lat.get_spins(), lat.read_accumulator()[0], lat.measure()["accept_rate"]))
+    (a, m, r), (b, n, s) = got
+    np.testing.assert_array_equal(a, b)
+    assert r == s
+    np.testing.assert_allclose(m, n, rtol=0, atol=1e-12 * max(1.0, np.abs(n).max()))
