@@ -722,8 +722,8 @@ int lattice_create(hs_lattice **out, int type, const int32_t dims[3], int period
     if (st == HS_OK && precision == HS_FP64) {
         // sin, cos(pi j / 4096) in units of 2^-63 for the FP64 trial's table lookup, from long double on the host
         const long double pi = 3.141592653589793238462643383279502884L;
-        std::vector<ulonglong2> tab(2048);
-        for (int j = 0; j < 2048; ++j) {
+        std::vector<ulonglong2> tab(1025);
+        for (int j = 0; j <= 1024; ++j) {
             const long double a = pi * (long double)j / 4096.0L;
             tab[j] = make_ulonglong2((unsigned long long)(sinl(a) * 0x1p63L + 0.5L),
                                      (unsigned long long)(cosl(a) * 0x1p63L + 0.5L));

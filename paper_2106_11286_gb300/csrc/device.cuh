@@ -87,9 +87,7 @@ __device__ __forceinline__ void sphere_fp64(uint4 w, double &x, double &y, doubl
 // ---- FP64 trial orientation in the integer pipe.  The FP64 pipe issues 2
 // instructions per cycle per SM, the integer units 32 (32x32->64 multiply) to
 // 128 (add, logic), so the sphere point is formed in 64-bit fixed point, about
-// 190 integer instructions, where FP64 took 26 that cost as much as 1600.
-// Every product keeps 61 bits or more below 1, so the results, rounded to
-// nearest, carry the error of that last rounding only.
+// 200 integer instructions, where FP64 took 26 that cost as much as 1600.
 //
 // floor(a b / 2^64), low partial product left out: at most 3 too small.
 __device__ __forceinline__ uint64_t mulhi_64(uint64_t a, uint64_t b) {
@@ -117,22 +115,34 @@ struct Trial64 {
     float fx, fy, fz;
 };
 
-// The sphere point of sphere_fp64 from one Philox block.
+// The sphere point of sphere_fp64 from one Philox block.  Small components carry
+// their digits too: r and a small sine keep an exponent of their own.
 //  * z = (iz - 2^52) 2^-52 exactly.
 //  * r = sqrt((1 - |z|)(1 + |z|)): both factors are exact integers; 1 - |z| is
 //    scaled up by an even power of two, so their product W lies in
 //    [1/16, 1/2); sqrt(W) starts from the hardware reciprocal square root
 //    (2^-22) and takes two Newton steps on the exact residual, W - Y^2 (2^-44,
-//    then below 2^-60).
-//  * phi = pi v = pi t - pi, t = iv 2^-52: sin and cos of pi t by quadrant,
-//    table and angle addition (Tang, "Table-lookup algorithms for elementary
-//    functions and their error analysis", 1991): 2048 entries of sin, cos
-//    (pi j / 4096) in units of 2^-63, then theta < pi/2 2^-11 by
-//    sin theta = theta - theta^3/6 (first omitted term 2^-58.6) and
-//    1 - cos theta = theta^2/2 - theta^4/24 (omitted 2^-71).
+//    then below 2^-60); the scale's root goes into the result's exponent.
+//  * phi = pi v = pi t - pi, t = iv 2^-52: sin and cos of pi t by octant, so
+//    that what may be small is a sine of an angle counted from its axis, table
+//    and angle addition (Tang, "Table-lookup algorithms for elementary functions
+//    and their error analysis", 1991): 1025 entries of sin, cos (pi j / 4096) in
+//    units of 2^-63, then theta < pi/2 2^-11 by sin theta = theta - theta^3/6
+//    (first omitted term 2^-58.6) and 1 - cos theta = theta^2/2 - theta^4/24
+//    (omitted 2^-71).  In the first step (one site of 1024) the sine is theta's
+//    own, from theta scaled up to 64 digits, with theta^5/120 (omitted term
+//    2^-74 of theta).
+// Against 128-bit arithmetic over 4 million words, most of them beside the poles
+// and axes, components are within 0.52 units in their last place from 1/2 to 1,
+// 1.2 above 2^-6, 3.2 above 2^-8 and 14 at any size; an FP64 form of this point
+// (2048 centred entries, theta^3 and theta^4) was off by up to 6.7 above 1/16,
+// 440 down to 2^-19, and by 2^-62 whatever the size below that.  With r and the
+// sines in fixed point alone the small components lost digits (570 units at
+// 2^-16, 5200 at 2^-19) for 3.5 % less time, 10 sweeps of 256^3 6.72 against 6.97
+// ms, 100 of 16^3 580 against 601 us.
 __device__ __forceinline__ Trial64 trial64(uint4 w, const ulonglong2 *tab) {
     Trial64 t;
-    const uint64_t one = 1ull << 52;
+    const uint64_t one = 1ull << 52, half_pi = 0xC90FDAA22168C235ull;  // pi/2 2^63
     const uint64_t iz = bits53(w.x, w.y), iv = bits53(w.z, w.w);
     const bool zneg = iz < one;
     const uint64_t m = zneg ? one - iz : iz - one;  // |z| 2^52
@@ -151,28 +161,40 @@ __device__ __forceinline__ Trial64 trial64(uint4 w, const ulonglong2 *tab) {
     const int64_t d0 = (int64_t)(int32_t)(E0 >> 12) * R;  // units of 2^-81
     const uint64_t Y1 = ((uint64_t)Y0 << 32) + (uint64_t)(d0 >> 17);
     const int32_t E1 = (int32_t)(uint32_t)(W - mulhi_64(Y1, Y1));
-    const uint64_t Y2 = Y1 + (uint64_t)(((int64_t)E1 * R) >> 29);
-    const uint64_t r = Y2 >> ((sh >> 1) - 5);  // units of 2^-62
+    const uint64_t r = Y1 + (uint64_t)(((int64_t)E1 * R) >> 29);  // units of 2^-(62 + rexp)
+    const int rexp = (sh >> 1) - 5;                               // 0 .. 26
 
     const uint32_t quad = (uint32_t)(iv >> 51);
-    const uint32_t j = (uint32_t)(iv >> 40) & 2047u;
+    const bool upper = (uint32_t)(iv >> 50) & 1u;  // the quadrant's upper octant: counted down from its end
+    const uint64_t g = upper ? (1ull << 51) - (iv & ((1ull << 51) - 1ull)) : iv & ((1ull << 50) - 1ull);
+    const uint32_t j = (uint32_t)(g >> 40);  // 0 .. 1024
     const ulonglong2 sc = __ldg(tab + j);
-    const uint64_t u = mulhi_64(iv << 24, 0xC90FDAA22168C235ull);  // theta 2^11, units of 2^-63 (pi/2 2^63)
-    const uint64_t s2 = mulhi_64(u, u);                            // theta^2 2^22, units of 2^-62
+    const uint64_t low = g << 24;
+    const uint64_t u = mulhi_64(low, half_pi);  // theta 2^11, units of 2^-63
+    const uint64_t s2 = mulhi_64(u, u);         // theta^2 2^22, units of 2^-62
     const uint32_t s2h = (uint32_t)(s2 >> 32);
     // (1 - cos theta) 2^23, units of 2^-62, and sin theta 2^11, units of 2^-63 (1/3 and 1/6 in 32 bits)
     const uint64_t c = s2 - ((uint64_t)__umulhi(__umulhi(s2h, s2h), 0x55555555u) << 10);
     const uint64_t sx = u - ((uint64_t)__umulhi(__umulhi(s2h, (uint32_t)(u >> 32)), 0x2AAAAAABu) << 12);
-    const uint64_t sn = sc.x + (mulhi_64(sc.y, sx) >> 10) - (mulhi_64(sc.x, c) >> 21);
+    uint64_t sn = sc.x + (mulhi_64(sc.y, sx) >> 10) - (mulhi_64(sc.x, c) >> 21);  // units of 2^-(63 + sexp)
     const uint64_t cs = sc.y - (mulhi_64(sc.x, sx) >> 10) - (mulhi_64(sc.y, c) >> 21);
+    int sexp = 0;
+    if (j == 0u) {  // theta (1 - theta^2/6 + theta^4/120), theta^2/6 and theta^4/120 in units of 2^-84
+        const int n = __clzll((long long)(low | 1ull << 24));  // 0 .. 39: low is a multiple of 2^24
+        const uint64_t U = mulhi_64(low << n, half_pi);
+        const uint64_t q = mulhi_64(s2, 0x2AAAAAAAAAAAAAABull) - ((uint64_t)__umulhi(__umulhi(s2h, s2h), 0x02222222u) << 12);
+        sn = U - (mulhi_64(U, q) >> 20);
+        sexp = 11 + n;
+    }
     // x = -r cos(pi t), y = -r sin(pi t)
-    const bool odd = quad & 1u;
-    const uint64_t X = mulhi_64(r, odd ? sn : cs), Y = mulhi_64(r, odd ? cs : sn);  // units of 2^-61
+    const bool swap = ((quad & 1u) != 0u) != upper;  // x takes the sine
+    const uint64_t X = mulhi_64(r, swap ? sn : cs), Y = mulhi_64(r, swap ? cs : sn);
+    const int xe = rexp + (swap ? sexp : 0), ye = rexp + (swap ? 0 : sexp);  // units of 2^-(61 + xe), 2^-(61 + ye)
     const bool xneg = quad == 0u || quad == 3u, yneg = quad < 2u;
-    t.x = fixed_to_double(X, 1024, xneg);
-    t.y = fixed_to_double(Y, 1024, yneg);
-    t.fx = (float)(uint32_t)(X >> 32) * 0x1p-29f;
-    t.fy = (float)(uint32_t)(Y >> 32) * 0x1p-29f;
+    t.x = fixed_to_double(X, 1024 - xe, xneg);
+    t.y = fixed_to_double(Y, 1024 - ye, yneg);
+    t.fx = (float)(uint32_t)(X >> 32) * __uint_as_float((uint32_t)(98 - xe) << 23);
+    t.fy = (float)(uint32_t)(Y >> 32) * __uint_as_float((uint32_t)(98 - ye) << 23);
     t.fx = xneg ? -t.fx : t.fx;
     t.fy = yneg ? -t.fy : t.fy;
     return t;

@@ -97,7 +97,7 @@ struct PassArgs {
     int tensor;             // 1: the on-site anisotropy tensor term is on
     double A[6];            // its symmetric tensor (xx, yy, zz, xy, xz, yz)
     float fA[6];
-    const ulonglong2 *sc_tab;  // FP64 trial: sin, cos(pi j / 4096) in units of 2^-63, j = 0..2047
+    const ulonglong2 *sc_tab;  // FP64 trial: sin, cos(pi j / 4096) in units of 2^-63, j = 0..1024
     int zaxis;              // 1: e = (0, 0, 1) exactly (the FP64 stencil takes S.e = S_z)
     uint32_t key0, key1, replica, sweep;
     float fdelta;           // FP64: bound on the error of the FP32 form of beta dH (decision_band); in what was
