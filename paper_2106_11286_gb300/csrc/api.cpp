@@ -678,6 +678,7 @@ int lattice_create(hs_lattice **out, int type, const int32_t dims[3], int period
     int st = HS_OK;
     Layout &L = h->L;
     L.structured = structured;
+    L.n_sm = h->n_sm;
     if (slab) {
         L.slab = true;
         L.z0 = slab->z0;

@@ -132,6 +132,7 @@ struct Layout {
     int ty;                 // z-march stencil: rows per plane-slab
     int order;              // register stencil: 1 ascending passes, 2 alternating (colour 1 descending)
     bool plain;             // register stencil: the ascending-only variant (lattices beyond 2^31 sites)
+    int n_sm;               // SMs of the lattice's device
     int n_colours;
     int64_t n_sites, n_present;
     // stencil

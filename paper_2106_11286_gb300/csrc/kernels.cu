@@ -1028,7 +1028,7 @@ const void *table_kernel_ptr(const Layout &L, bool meas) {
     if constexpr (P == HS_FP64) {
         int64_t most = 0;  // sites of the largest class
         for (int c = 0; c < L.n_colours; ++c) most = std::max(most, L.colour_begin[c + 1] - L.colour_begin[c]);
-        if (most > 152 * kBlock) return table_variant<P, 0, false, true>(meas);
+        if (most > (int64_t)L.n_sm * kBlock) return table_variant<P, 0, false, true>(meas);
     }
     return table_variant<P, 0, false>(meas);
 }
@@ -1405,7 +1405,7 @@ static cudaError_t scatter_p(const Layout &L, double *xyz, cudaStream_t s) {
 template <int P, int V>
 static cudaError_t export_v(const Layout &L, double *xyz, cudaStream_t s) {
     const int64_t n_vec = (int64_t)L.nz * L.Ly * (L.Lh / V);
-    sc_export_kernel<P, V><<<grid_for(n_vec, 152 * 8), kBlock, 0, s>>>(
+    sc_export_kernel<P, V><<<grid_for(n_vec, L.n_sm * 8), kBlock, 0, s>>>(
         L.planes, xyz, L.Ly, (int64_t)L.Lz * L.Ly * L.Lh, L.Lh, L.slab ? 1 : 0, L.z0, FastDiv((uint32_t)(L.Lh / V)),
         FastDiv((uint32_t)L.Ly), (uint32_t)n_vec, (uintptr_t)xyz % 16 == 0 ? 1 : 0);
     return cudaGetLastError();
