@@ -43,11 +43,11 @@ __global__ void __launch_bounds__(kClusterThreads, 1) sc_cluster_kernel(const Pa
                                               (int)gridDim.x);
 }
 
+// (Always ascending: a warp's items and their sum are the same in either direction.)
 template <int P, int V, bool MEAS, int AX>
 __global__ void __launch_bounds__(kClusterThreads, 1) sc_slab_kernel(const PassArgs args, void *planes, int n_sweeps,
-                                                                     int alternate, int depth) {
+                                                                     int depth) {
     pdl_enter();
-    (void)alternate;  // a warp's items and their sum are the same in either direction
     sweep_slabs<P, V, MEAS, AX>(args, planes, n_sweeps, depth, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -61,29 +61,38 @@ __global__ void __launch_bounds__(kBlock, 2) sc_grid_kernel(const PassArgs args,
 
 // The variants of one precision and width: the tensor term, or FP32's S.e = S_z.
 template <int P, int V, bool MEAS>
-const void *group_ptr(GroupKind kind, bool ten, bool ax) {
-    const bool grid = kind == kGroupGrid;
-    if (kind == kGroupSlabs) {
-        if constexpr (P == HS_FP32)
-            if (ax) return (const void *)sc_slab_kernel<P, V, MEAS, 1>;
-        return (const void *)sc_slab_kernel<P, V, MEAS, 0>;
-    }
-    if (ten)
-        return grid ? (const void *)sc_grid_kernel<P, V, MEAS, 0, true> : (const void *)sc_cluster_kernel<P, V, MEAS, 0, true>;
+const void *grid_ptr(bool ten, bool ax) {
+    if (ten) return (const void *)sc_grid_kernel<P, V, MEAS, 0, true>;
+    if constexpr (P == HS_FP32)
+        if (ax) return (const void *)sc_grid_kernel<P, V, MEAS, 1, false>;
+    return (const void *)sc_grid_kernel<P, V, MEAS, 0, false>;
+}
+
+template <int P, int V, bool MEAS>
+const void *cluster_ptr(GroupKind kind, bool ten, bool ax) {
+    const bool slabs = kind == kGroupSlabs;
+    if (ten) return slabs ? nullptr : (const void *)sc_cluster_kernel<P, V, MEAS, 0, true>;
     if constexpr (P == HS_FP32)
         if (ax)
-            return grid ? (const void *)sc_grid_kernel<P, V, MEAS, 1, false>
-                        : (const void *)sc_cluster_kernel<P, V, MEAS, 1, false>;
-    return grid ? (const void *)sc_grid_kernel<P, V, MEAS, 0, false> : (const void *)sc_cluster_kernel<P, V, MEAS, 0, false>;
+            return slabs ? (const void *)sc_slab_kernel<P, V, MEAS, 1> : (const void *)sc_cluster_kernel<P, V, MEAS, 1, false>;
+    return slabs ? (const void *)sc_slab_kernel<P, V, MEAS, 0> : (const void *)sc_cluster_kernel<P, V, MEAS, 0, false>;
+}
+
+template <int P, int V, bool MEAS>
+const void *group_ptr(GroupKind kind, bool ten, bool ax) {
+    if (kind == kGroupGrid) return grid_ptr<P, V, MEAS>(ten, ax);
+    if constexpr (P != HS_FP64 || V == 1)  // FP64 clusters take one site a thread
+        return cluster_ptr<P, V, MEAS>(kind, ten, ax);
+    return nullptr;
 }
 
 template <int P>
-const void *group_vec(int vec, bool meas, GroupKind grid, bool ten, bool ax) {
+const void *group_vec(int vec, bool meas, GroupKind kind, bool ten, bool ax) {
     switch (vec) {
-    case 1: return meas ? group_ptr<P, 1, true>(grid, ten, ax) : group_ptr<P, 1, false>(grid, ten, ax);
-    case 2: return meas ? group_ptr<P, 2, true>(grid, ten, ax) : group_ptr<P, 2, false>(grid, ten, ax);
+    case 1: return meas ? group_ptr<P, 1, true>(kind, ten, ax) : group_ptr<P, 1, false>(kind, ten, ax);
+    case 2: return meas ? group_ptr<P, 2, true>(kind, ten, ax) : group_ptr<P, 2, false>(kind, ten, ax);
     case 4:
-        if constexpr (P != HS_FP64) return meas ? group_ptr<P, 4, true>(grid, ten, ax) : group_ptr<P, 4, false>(grid, ten, ax);
+        if constexpr (P != HS_FP64) return meas ? group_ptr<P, 4, true>(kind, ten, ax) : group_ptr<P, 4, false>(kind, ten, ax);
         break;
     default: break;
     }
@@ -233,8 +242,9 @@ cudaError_t launch_group(int precision, const Layout &L, const GroupPlan &p, con
     cudaLaunchAttribute attr[2];
     group_config(cfg, attr, precision, p, s);
     int depth = p.depth;
+    void *slabs[] = {&args, &planes, &n_sweeps, &depth};
     void *params[] = {&args, &planes, &n_sweeps, &alternate, &depth, &arrivals};  // a cluster's kernel takes the first five
-    return cudaLaunchKernelExC(&cfg, k, params);
+    return cudaLaunchKernelExC(&cfg, k, p.kind == kGroupSlabs ? slabs : params);
 }
 
 }  // namespace hs
