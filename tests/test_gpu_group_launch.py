@@ -1,6 +1,8 @@
 """Which launch runs a small lattice's sweeps (hs_get_group_launch), and that
 the configuration calls leave it as it was where they say that they change
 nothing."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -105,3 +107,37 @@ def test_the_largest_groups_equal_the_chain(kind, dims, precision):
     np.testing.assert_array_equal(a, b)
     assert r == s
     np.testing.assert_allclose(m, n, rtol=0, atol=1e-12 * max(1.0, np.abs(n).max()))
+
+
+def test_lattices_side_by_side():
+    """Every kind of launch at once, each lattice on a thread and a stream of its own: the chains that they have alone."""
+    made = [("sc", (16, 16, 16), "fp64"), ("sc", (20, 16, 6), "fp64"), ("sc", (48, 48, 48), "fp32"), ("sc", (96, 96, 96), "fp32"),
+            ("bcc", (20, 20, 20), "fp32"), ("fcc", (12, 12, 12), "fp64"), ("sc", (32, 32, 32), "fp16"), ("bcc", (40, 40, 40), "fp32")]
+
+    def swept(lat):
+        lat.init()
+        lat.accumulate(True)
+        lat.sweep(0.8, 130)
+        return lat.get_spins(), lat.read_accumulator()
+
+    def lattice(k, **kw):
+        kind, dims, precision = made[k]
+        return hs.Lattice(kind, dims=dims, precision=precision, seed=k, K=0.1, **kw)
+
+    got, lats = [None] * len(made), [lattice(k, stream=torch.cuda.Stream()) for k in range(len(made))]
+
+    def work(k):
+        got[k] = swept(lats[k])
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(made))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for k in range(len(made)):
+        lats[k].close()
+        with lattice(k) as lat:
+            spins, (moments, count) = swept(lat)
+        np.testing.assert_array_equal(got[k][0], spins)
+        assert got[k][1][1] == count == 130
+        np.testing.assert_allclose(got[k][1][0], moments, rtol=0, atol=1e-12 * np.abs(moments).max())
